@@ -354,8 +354,8 @@ class _Mesh:
         X = x[el]                                                            # [E, d+1, d]
         self.X0, self.E = X[:, 0], X.shape[0]
         self.J = (X[:, 1:] - X[:, :1]).transpose(1, 2).contiguous()
-        self.det = torch.linalg.det(self.J)
-        self.Jinv = torch.linalg.inv(self.J)
+        J = self.J.cpu()
+        self.det, self.Jinv = torch.linalg.det(J).to(device), torch.linalg.inv(J).to(device)
         far, P, out = [], [], []
         for f in range(d + 1):
             own = [j for j in range(d + 1) if j != f]
