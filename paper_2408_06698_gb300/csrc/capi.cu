@@ -315,7 +315,7 @@ void convert(const std::vector<double>& src, std::vector<unsigned char>& dst, si
 }
 
 // Reorder the host FP64 tables into the kernel layouts (see hopu_internal.h).
-constexpr int kNumTables = 14;
+constexpr int kNumTables = 16;
 
 // Row stride of the point-major tables: an odd multiple of 16 bytes (matches
 // row_stride<T> in kernels.cuh).
@@ -379,6 +379,26 @@ void kernel_tables(const RefTables& R, bool fp64, std::vector<std::vector<double
       WPsi[(size_t)m * nqf + q] = R.wf[q] * R.psi[(size_t)q * nf + m];
     }
   Wf = R.wf;
+  // the facet basis at the collapsed points as products of one-dimensional factors: A_p the
+  // orthonormal Legendre polynomial of the first direction, B_m = psi_m / A_p taken where
+  // |A_p| is largest (a constant along the first direction)
+  auto& FacA = out[14];
+  auto& FacB = out[15];
+  const int mf = rule_m(3 * R.k), K1 = R.k + 1;
+  std::vector<double> t1, w1;
+  gauss_jacobi01(mf, 0, t1, w1);
+  FacA.assign((size_t)mf * K1, 0.0);
+  FacB.assign((size_t)mf * nf, 1.0);
+  for (int i = 0; i < mf; ++i) dubiner(1, R.k, &t1[i], &FacA[(size_t)i * K1], nullptr);
+  if (d == 3)
+    for (int n = 0, m = 0; n <= R.k; ++n)
+      for (int p = 0; p <= n; ++p, ++m) {
+        int best = 0;
+        for (int i = 1; i < mf; ++i)
+          if (std::fabs(FacA[(size_t)i * K1 + p]) > std::fabs(FacA[(size_t)best * K1 + p])) best = i;
+        for (int j = 0; j < mf; ++j)
+          FacB[(size_t)j * nf + m] = R.psi[(size_t)(best * mf + j) * nf + m] / FacA[(size_t)best * K1 + p];
+      }
   // n_loc x n_loc tables for the projection GEMMs, [s][r] with rows padded to nlp
   const int nlp = (nl + 3) / 4 * 4;
   DinvT.assign((size_t)nl * nlp, 0.0);
@@ -925,7 +945,7 @@ hopu_status create_impl(const hopu_mesh_desc* mesh, const hopu_options* opts, vo
   const void** slots[kNumTables] = {&c->dt.Bt,   &c->dt.Wq,  &c->dt.Dm,    &c->dt.TrM,
                                     &c->dt.TrP,  &c->dt.Psi, &c->dt.WPsi,  &c->dt.Wf,
                                     &c->dt.DinvT, &c->dt.DT, &c->dt.Dinv, &c->dt.Drow, &c->dt.Dn,
-                                    &c->dt.dBt};
+                                    &c->dt.dBt, &c->dt.FacA, &c->dt.FacB};
   for (int i = 0; i < kNumTables; ++i) *slots[i] = tb + offs[i];
   if (!c->fp64) {
     std::vector<float> csr;

@@ -40,6 +40,9 @@ struct DevTabs {
   const void* Psi = nullptr;    // [nf][nqf]       psi_m(s_q)
   const void* WPsi = nullptr;   // [nf][nqf]       w_q psi_m(s_q)
   const void* Wf = nullptr;     // [nqf]           facet weights
+  const void* FacA = nullptr;   // [mf][k+1]       facet basis factors at the points (t_i, t_j) of the facet
+  const void* FacB = nullptr;   // [mf][nf]          rule: psi_m = A_p(t_i) B_m(t_j), p the first index of
+                                //                 mode m (2D: psi_p = A_p, B = 1)
   const void* DinvT = nullptr;  // [nloc][nlp]     DinvT[s][r] = Dinv[r][s]  (nlp = nloc rounded up to 4)
   const void* Dcsr = nullptr;   // FP32: the nonzeros of D by rows, 16-byte entries (layout in
                                 //   k_v2l / warp_tile_residual); csr_n entries in all

@@ -23,8 +23,11 @@ template <int D, int K>
 struct FacAR {
   using F = FacR<D, K>;
   static constexpr int NB = F::NB, NF = F::NF, NL = F::NL, NQF = F::NQF, FPW = F::FPW, WARPS = 4;
-  static constexpr int NB4 = F::NB4, NF4 = F::NF4;
-  static constexpr size_t SMEM = F::SMEM;        // the tables of k_facet_r
+  static constexpr int NB4 = F::NB4, NF4 = r4i(NF);
+  static constexpr int O_TRM = 0;                                // [(D+1) NF][NB4]
+  static constexpr int O_PSI = O_TRM + (D + 1) * NF * NB4;       // [NQF][NF4]   psi_m(s_q)
+  static constexpr int O_WPSI = O_PSI + NQF * NF4;               // [NQF][NF4]   w_q psi_m(s_q)
+  static constexpr size_t SMEM = size_t(O_WPSI + NQF * NF4) * 4;
   static constexpr int REGS = 2 * NB + 8 * NF;   // coefficients of one field, modal vectors, moments
   static constexpr bool OK = REGS <= 200;
   static constexpr int MINB = REGS <= 110 ? 3 : 2;
@@ -35,7 +38,6 @@ __global__ void __launch_bounds__(32 * FacAR<D, K>::WARPS, FacAR<D, K>::MINB)
     k_facet_adj_r(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ ybar, int lconst,
                   const int8_t* __restrict__ facet_l, float* __restrict__ gamU, float* __restrict__ gamW) {
   using C = FacAR<D, K>;
-  using FR = FacR<D, K>;
   constexpr int NB = C::NB, NF = C::NF, NL = C::NL, NQF = C::NQF, NB4 = C::NB4, NF4 = C::NF4, FPW = C::FPW;
   constexpr int GT = Shape<D, K>::gt;
   extern __shared__ __align__(16) float sm[];
@@ -44,21 +46,19 @@ __global__ void __launch_bounds__(32 * FacAR<D, K>::WARPS, FacAR<D, K>::MINB)
     const float* TrMg = static_cast<const float*>(tb.TrM);
     const float* Psig = static_cast<const float*>(tb.Psi);    // [NF][NQF]
     const float* WPsig = static_cast<const float*>(tb.WPsi);  // [NF][NQF]
-    const float* Wfg = static_cast<const float*>(tb.Wf);
     for (int t = threadIdx.x; t < (D + 1) * NF * NB4; t += blockDim.x) {
       const int row = t / NB4, i = t - row * NB4;
-      sm[FR::O_TRM + t] = i < NB ? TrMg[row * NB + i] : 0.0f;
+      sm[C::O_TRM + t] = i < NB ? TrMg[row * NB + i] : 0.0f;
     }
     for (int t = threadIdx.x; t < NQF * NF4; t += blockDim.x) {
       const int q = t / NF4, mm = t - q * NF4;
-      sm[FR::O_PSI + t] = mm < NF ? Psig[mm * NQF + q] : 0.0f;
-      sm[FR::O_WPSI + t] = mm < NF ? WPsig[mm * NQF + q] : 0.0f;
+      sm[C::O_PSI + t] = mm < NF ? Psig[mm * NQF + q] : 0.0f;
+      sm[C::O_WPSI + t] = mm < NF ? WPsig[mm * NQF + q] : 0.0f;
     }
-    for (int t = threadIdx.x; t < NQF; t += blockDim.x) sm[FR::O_WF + t] = Wfg[t];
   }
-  const float* sTrM = sm + FR::O_TRM;
-  const float* sPsi = sm + FR::O_PSI;
-  const float* sWPsi = sm + FR::O_WPSI;
+  const float* sTrM = sm + C::O_TRM;
+  const float* sPsi = sm + C::O_PSI;
+  const float* sWPsi = sm + C::O_WPSI;
   pdl_wait();
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

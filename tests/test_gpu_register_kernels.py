@@ -1,0 +1,66 @@
+"""The register-resident FP32 kernels over every order, against the FP64 oracle.
+
+Small meshes whose facet and element counts are no multiple of a warp's share, so that the
+last group of every launch is ragged and element records start at every offset modulo 16
+bytes; random data and per-facet orders; walls and inlets; a wind of its own and w = u.
+Tolerance: the stated FP32 bound of the operator, 1e-6 of the largest output.
+"""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from oracle import convection as C
+from oracle import fe, hdiv, mesh
+
+pytestmark = pytest.mark.gpu
+
+ORDERS = [(2, 3, 1), (2, 5, 2), (2, 4, 3), (2, 3, 4), (3, 3, 1), (3, 4, 2), (3, 3, 3), (3, 3, 4), (3, 3, 5)]
+
+
+def _rel(got, ref):
+    got = got.detach().double().cpu().numpy().reshape(-1)
+    return float(np.abs(got - np.asarray(ref).reshape(-1)).max() / np.abs(ref).max())
+
+
+def _setup(dim, n, k, walls):
+    from paper_2408_06698_gb300 import Hopu
+    m = W.periodic_box_mesh(dim, n)
+    rep = None if walls else m.rep
+    g = Hopu(m.coords, m.elems, rep, k=k, l=k - 1, prec="f32")
+    topo = mesh.MeshTopo(m.coords, m.elems, rep)
+    return g, topo, fe.ref_element(dim, k)
+
+
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("dim,n,k", ORDERS)
+def test_apply_every_order(dim, n, k, walls):
+    g, topo, ref = _setup(dim, n, k, walls)
+    rng = np.random.default_rng(7000 + 100 * dim + 10 * k + walls)
+    sp = hdiv.HDiv(topo, ref)
+    f32 = lambda x: x.astype(np.float32).astype(np.float64)  # noqa: E731
+    wV = f32(rng.standard_normal(sp.n_hdiv))
+    w = sp.to_l2(wV)
+    u = f32(sp.to_l2(rng.standard_normal(sp.n_hdiv)))  # its own wind below: normal-continuous
+    fl = rng.integers(-1, k + 1, size=topo.n_facets).astype(np.int8)
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x).reshape(-1), dtype=torch.float32, device=g.device)  # noqa: E731
+    exterior = inlet = None
+    if walls:
+        b = np.where(topo.boundary)[0][::3]
+        vals = rng.standard_normal((1, 1, dim)) * np.ones((b.size, ref.wf.size, 1))   # constant per facet: exact modes
+        g.set_inlet(b, vals)
+        inlet = np.zeros(topo.n_facets, dtype=bool)
+        inlet[b] = True
+        ext_u = np.zeros((topo.n_facets, ref.wf.size, dim))
+        ext_u[b] = vals
+    for wind, same in ((w, False), (u, True)):
+        if walls:
+            exterior = (ext_u, C.facet_trace(topo, ref, wind, "A"))
+        gu, gw = dev(u), dev(wV)
+        apply = (lambda: g.apply_convection_l2(gu, gu)) if same else (lambda: g.apply_convection(gw, gu))
+        g.set_facet_l(None)
+        y = apply()
+        assert _rel(y, C.apply(topo, ref, wind, u, k - 1, exterior=exterior, inlet=inlet)) < 1e-6
+        g.set_facet_l(torch.as_tensor(fl, device=g.device))
+        y = apply()
+        assert _rel(y, C.apply(topo, ref, wind, u, fl.astype(np.int64), exterior=exterior, inlet=inlet)) < 1e-6
