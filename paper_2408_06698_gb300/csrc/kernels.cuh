@@ -21,6 +21,12 @@ __host__ __device__ constexpr int cbinom(int n, int r) {
   return (r < 0 || n < r) ? 0 : v;
 }
 __host__ __device__ constexpr int cnbasis(int dim, int k) { return k < 0 ? 0 : cbinom(k + dim, dim); }
+// total degree of the m-th function of the graded orthonormal basis of P^k in dimension d
+__host__ __device__ constexpr int mode_degree(int d, int m) {
+  int n = 0;
+  while (cnbasis(d, n) <= m) ++n;
+  return n;
+}
 __host__ __device__ constexpr int cpow(int b, int e) { return e == 0 ? 1 : b * cpow(b, e - 1); }
 __host__ __device__ constexpr int r4i(int n) { return ((n + 3) / 4) * 4; }
 

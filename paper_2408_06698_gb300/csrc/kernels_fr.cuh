@@ -40,13 +40,6 @@
 
 namespace hopu {
 
-// total degree of the m-th function of the graded orthonormal basis of P^k in dimension d
-__host__ __device__ constexpr int mode_degree(int d, int m) {
-  int n = 0;
-  while (cnbasis(d, n) <= m) ++n;
-  return n;
-}
-
 template <int D, int K>
 struct FacR {
   using S = Shape<D, K>;
@@ -111,8 +104,6 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
   const float* sA = sm + C::O_A;
   const float* sB = sm + C::O_B;
   const float* sWf = sm + C::O_WF;
-  pdl_wait();
-  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* sRec = sm + C::O_REC + warp * 2 * FPW * RST;
   const double* sGeo = reinterpret_cast<const double*>(sm + C::O_GEO + warp * C::GEO);
@@ -204,10 +195,10 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
       if (i0 + t < end) cp_async<8>(const_cast<double*>(sGeo) + t, m.fgeo + i0 + t);
   };
   sides(grp);
-  if (grp < ngroups) {
-    request_geo(grp);
-    request(uL, npa, npb);
-  }
+  if (grp < ngroups) request_geo(grp);  // mesh data: before the wait for the previous kernel
+  pdl_wait();
+  __syncthreads();
+  if (grp < ngroups) request(uL, npa, npb);
   for (; grp < ngroups; grp += gstep) {
     const int64_t F0 = grp * FPW;
     const bool act = lane_on && F0 + fl < m.NF;

@@ -4,17 +4,19 @@
 // A warp takes ELW = 32 / D elements and a lane owns one (element, component a) pair: the
 // coefficients c of u_a, its modal reference gradients G_c = Dm_c c (c < D, dim P^{k-1}
 // entries each) and the accumulators r of its test integrals stay in registers for the whole
-// element.  The quadrature points are walked in the same order by every lane, so the basis
-// row phi(x_q) is one broadcast shared-memory load for the whole warp; per point a lane forms
+// element, as pairs of neighbouring basis indices (f32x2.cuh).  The quadrature points are
+// walked in the same order by every lane, so the basis row phi(x_q) is one broadcast
+// shared-memory load for the whole warp; per point a lane forms
 //   u_a = sum_i phi_i c_i,   d^_c u_a = sum_j phi_j G_c[j],
-// its shares M[c][a] u_a of W_c = sum_b M[c][b] u_b (M = |det J| J^-1, so W = |det J| J^-1 u)
-// and sum_c M[c][a] d^_c u_a of div^ W, sums them over the D lanes of its element with
-// shuffles, and adds f_a = w_q (div^W u_a + W . grad^ u_a) phi_i to r_i (the element-wise
-// integration by parts of the conservative form, as the other volume kernels).  The facet
-// lift sum_fm TrM[fm][i] gam[e][fm][a] and 1/|det J| follow; the outputs leave through a
-// per-warp staging buffer with coalesced stores.  Compared with one warp per element (lanes
-// on quadrature points, coefficient rows read from shared memory per point) this moves the
-// contractions from the shared-memory pipe into registers.
+// takes the other components' u from its element's lanes (two shuffles) for W = M u
+// (M = |det J| J^-1), sums its share sum_c M[c][a] d^_c u_a of div^ W over them, and adds
+// f_a = w_q (div^W u_a + W . grad^ u_a) phi_i to r_i (the element-wise integration by parts of
+// the conservative form, as the other volume kernels).  The facet lift
+// sum_fm TrM[fm][i] gam[e][fm][a] and 1/|det J| follow; the outputs leave through a per-warp
+// staging buffer with coalesced stores.  Differentiation lowers the degree and a trace does
+// not raise it: Dm[c][j][i] = 0 for deg phi_j >= deg phi_i and TrM[m][i] = 0 for
+// deg psi_m > deg phi_i, and both products run over the rest only.  The group's records
+// arrive by cp.async, requested one group ahead.
 //
 // GTAB: the reference gradients at the points come from staged tables of d phi_i / d xhat_c
 // instead of the modal gradients G held in registers (d n_{b,k-1} fewer registers, more
@@ -26,15 +28,30 @@
 // keeps component b in registers), ell = D chat (every lane forms its component's share of
 // each row, D staged per CTA, the shares summed by shuffles); interior rows are combined
 // into the V_h output, facet rows go to lf with the sign sigma.
+//
+// WSEP: a wind w of its own: lane a holds the modal coefficients of the reference component
+// W_a = sum_b M[a][b] w_b and those of div^ W = sum_a d^_a W_a (summed over the element's lanes
+// once), evaluates both at the points with the same basis row and takes the other W by
+// shuffles; one point per pass where the registers end (k = 4).
+//
+// Bound: the FMA units' register reads (three distinct 64-bit operands per paired FMA: a copy
+// of the inner loop alone ran at 210 cycles per point and warp at k = 4, against 139 of FMA
+// issue, whether the rows came once or twice from shared memory).  Measured (CUDA events, per
+// launch): 32^3 x 6, k = 4, w = u 629 -> 528 us (scalar FMAs, dense Dm and TrM products and
+// strided coefficient loads before), separate wind 1815 -> 761 us (a warp per element before;
+// the basis split over two lanes 1054 us); 24^3 x 6, k = 3, w = u 90 -> 84 us; 16^3 x 6, k = 3,
+// separate wind 57 -> 37 us.
 #pragma once
+#include "f32x2.cuh"
 #include "kernels.cuh"
 
 namespace hopu {
 
-template <int D, int K, bool GTAB = false>
+template <int D, int K, bool GTAB = false, bool WSEP = false>
 struct VolR {
   using S = Shape<D, K>;
   static constexpr int NB = S::nb, NB1 = cnbasis(D, K - 1), NF = S::nf, NL = S::nloc, NQ = S::nq, GT = S::gt;
+  static constexpr int NP = (NB + 1) / 2, NP1 = (NB1 + 1) / 2;  // pairs of basis indices
   static constexpr int ELW = 32 / D;                 // elements per warp
   static constexpr int WARPS = GTAB ? 6 : 4;
   static constexpr int NBQ = row_stride<float>(NB);  // Bt rows (point-major, as in global memory)
@@ -45,28 +62,42 @@ struct VolR {
   static constexpr int O_DM = r4i(O_WQ + NQ);
   static constexpr int O_TRM = O_DM + (GTAB ? 0 : D * NB1 * NB4);
   static constexpr int O_W = O_TRM + (D + 1) * NF * NB4;
-  static constexpr int PER_WARP = r4i(ELW * NL);     // output staging of the warp's elements
-  static constexpr int GW = r4i(ELW * NG);           // the warp's facet moments, staged by cp.async
-  static constexpr int O_G = O_W + WARPS * PER_WARP;
+  static constexpr int PER_WARP = r4i(ELW * NL);     // the warp's element records: in, and out
+  static constexpr int GW = r4i(ELW * NG);           // the warp's facet moments
+  static constexpr int O_G = O_W + WARPS * (WSEP ? 3 : 2) * PER_WARP;
   static constexpr size_t SMEM = size_t(O_G + WARPS * GW) * 4;
   static constexpr int NLR = row_stride<float>(NL);  // rows of the row-major D in global memory
   static constexpr int NDP = D * NB4;                // fused back-projection: D [NL][D blocks of NB4]
   static constexpr int O_D = O_G + WARPS * GW;
   static constexpr size_t SMEM_FUSE = size_t(O_D + NL * NDP) * 4;
-  static constexpr int REGS = 2 * NB + (GTAB ? 0 : D * NB1);  // c, r (and G) of a lane
-  static constexpr int MINB = GTAB ? 2 : (REGS <= 100 ? 3 : 2);  // resident CTAs asked of the register allocator
-  static constexpr bool OK = REGS <= 140 && SMEM <= 200 * 1024;
+  static constexpr int REGS = (WSEP ? 3 * NB + NB1 : 2 * NB) + (GTAB ? 0 : D * NB1);  // c, r, G of a lane (and w, div w)
+  static constexpr int XP = REGS <= 140 ? 2 : 1;  // quadrature points per pass
+  static constexpr int MINB = GTAB ? 2 : (REGS <= 90 ? 3 : 2);  // resident CTAs asked of the register allocator
+  static constexpr bool OK = REGS <= 190 && SMEM <= 200 * 1024;
   static constexpr bool FUSE_OK = OK && SMEM_FUSE <= 200 * 1024;
 };
 
-template <int D, int K, bool FUSE, bool GTAB>
-__global__ void __launch_bounds__(32 * VolR<D, K, GTAB>::WARPS, VolR<D, K, GTAB>::MINB)
-    k_volume_r(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ gam, float* out,
-               Combine cmb, float* __restrict__ lf) {
-  using C = VolR<D, K, GTAB>;
+// A warp copies the records of ne consecutive elements (NV values each) starting at element e0.
+template <int NV, int GROUP>
+__device__ __forceinline__ void warp_copy_records(float* dst, const float* src, int64_t e0, int ne, int lane) {
+  constexpr int CH = gcd_pow2(GROUP * NV * 4);  // a whole group starts on a multiple of its size
+  const char* s = reinterpret_cast<const char*>(src + e0 * NV);
+  char* d = reinterpret_cast<char*>(dst);
+  if (ne == GROUP) {
+    for (int t = lane; t < GROUP * NV * 4 / CH; t += 32) cp_async<CH>(d + t * CH, s + t * CH);
+  } else {
+    for (int t = lane; t < ne * NV; t += 32) cp_async<4>(d + 4 * t, s + 4 * t);
+  }
+}
+
+template <int D, int K, bool FUSE, bool GTAB, bool WSEP>
+__global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K, GTAB, WSEP>::MINB)
+    k_volume_r(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ wL,
+               const float* __restrict__ gam, float* out, Combine cmb, float* __restrict__ lf) {
+  using C = VolR<D, K, GTAB, WSEP>;
   using S = Shape<D, K>;
   constexpr int NB = C::NB, NB1 = C::NB1, NF = C::NF, NL = C::NL, NQ = C::NQ, GT = C::GT;
-  constexpr int NBQ = C::NBQ, NB4 = C::NB4, NG = C::NG, ELW = C::ELW;
+  constexpr int NBQ = C::NBQ, NB4 = C::NB4, NG = C::NG, ELW = C::ELW, NP = C::NP, NP1 = C::NP1;
   extern __shared__ __align__(16) float sm[];
   pdl_trigger();
   {
@@ -106,180 +137,271 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB>::WARPS, VolR<D, K, GTAB>
   const bool lane_on = lane < D * ELW;
   const int el = lane_on ? lane / D : 0;
   const int a = lane_on ? lane - el * D : 0;
+  const int a1 = (a + 1) % D, a2 = (a + 2) % D;
   // the other lanes of the element (idle lanes talk to themselves)
-  const int p1 = lane_on ? el * D + (a + 1) % D : lane;
-  const int p2 = lane_on ? el * D + (a + 2) % D : lane;
-  float* sY = sm + C::O_W + warp * C::PER_WARP;
+  const int p1 = lane_on ? el * D + a1 : lane;
+  const int p2 = lane_on ? el * D + a2 : lane;
+  float* sIn = sm + C::O_W + warp * (WSEP ? 3 : 2) * C::PER_WARP;
+  float* sY = sIn + C::PER_WARP;
+  float* sWn = sY + (WSEP ? C::PER_WARP : 0);  // the wind's records (WSEP)
   float* sG = sm + C::O_G + warp * C::GW;
-  const int64_t ngroups = (m.E + ELW - 1) / ELW;
-  for (int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x; grp < ngroups; grp += (int64_t)gridDim.x * C::WARPS) {
+  const int64_t ngroups = (m.E + ELW - 1) / ELW, gstep = (int64_t)gridDim.x * C::WARPS;
+  auto count = [&](int64_t g) { return (m.E - g * ELW < ELW) ? (int)(m.E - g * ELW) : ELW; };
+  int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x;
+  auto request = [&](int64_t g) {
+    warp_copy_records<NL, ELW>(sIn, uL, g * ELW, count(g), lane);
+    if (WSEP) warp_copy_records<NL, ELW>(sWn, wL, g * ELW, count(g), lane);
+  };
+  if (grp < ngroups) request(grp);
+  cp_commit();
+  for (; grp < ngroups; grp += gstep) {
     const int64_t e0 = grp * ELW;
-    const int ne = (m.E - e0 < ELW) ? (int)(m.E - e0) : ELW;
+    const int ne = count(grp);
     const bool act = lane_on && el < ne;
     const int64_t e = act ? e0 + el : e0;  // inactive lanes read the group's first element
-    // the group's facet moments arrive in shared memory while the points are walked
-    for (int k2 = 0; k2 < ne; ++k2) warp_copy_async<NG * 4>(sG + k2 * NG, gam + (e0 + k2) * NG, lane);
-    cp_commit();
-    float c[NB];
-    {
-      const float* up = uL + e * NL + a * NB;
-#pragma unroll
-      for (int i = 0; i < NB; ++i) c[i] = __ldg(up + i);
-    }
     const double* gp = m.geoT + e * GT;
-    float Mcol[D];  // column a of M = |det J| J^-1
+    // M = |det J| J^-1: its columns a, a + 1, a + 2 (w = u), or its row a in M0 (separate wind)
+    float M0[D], M1[WSEP ? 1 : D], M2[WSEP ? 1 : D];
 #pragma unroll
-    for (int cc = 0; cc < D; ++cc) Mcol[cc] = float(__ldg(gp + 2 * D * D + cc * D + a));
+    for (int cc = 0; cc < D; ++cc) {
+      M0[cc] = float(__ldg(gp + 2 * D * D + (WSEP ? a * D + cc : cc * D + a)));
+      if constexpr (!WSEP) {
+        M1[cc] = float(__ldg(gp + 2 * D * D + cc * D + a1));
+        M2[cc] = D == 3 ? float(__ldg(gp + 2 * D * D + cc * D + a2)) : 0.0f;
+      }
+    }
     const float invabs = float(__ldg(gp + 3 * D * D));
-    // modal reference gradients of u_a: G[cc][j] = sum_i Dm[cc][j][i] c_i (not with GTAB)
-    constexpr int NG1 = GTAB ? 1 : NB1;
-    float G[D][NG1];
+    f2 c[NP], cw[WSEP ? NP : 1];
+    cp_wait<0>();
+    __syncwarp();
+    {
+      const int o = ((act ? el : 0) * D + a) * NB;
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        c[j] = f2_pack(sIn[o + 2 * j], 2 * j + 1 < NB ? sIn[o + 2 * j + 1] : 0.0f);
+        if constexpr (WSEP) {  // modal W_a = sum_b M[a][b] w_b, the wind's reference component a
+          float v[2] = {0.0f, 0.0f};
+#pragma unroll
+          for (int w = 0; w < 2; ++w)
+            if (2 * j + w < NB) {
+#pragma unroll
+              for (int b = 0; b < D; ++b) v[w] = fmaf(M0[b], sWn[((act ? el : 0) * D + b) * NB + 2 * j + w], v[w]);
+            }
+          cw[j] = f2_pack(v[0], v[1]);
+        }
+      }
+    }
+    __syncwarp();
+    // this group's facet moments and the next group's coefficients arrive during the points
+    warp_copy_records<NG, ELW>(sG, gam, e0, ne, lane);
+    if (grp + gstep < ngroups) request(grp + gstep);
+    cp_commit();
+    // entry `row` of the modal reference derivative Dm_cc of the coefficients x
+    auto derivative = [&](const f2 (&x)[NP], int cc, int row) -> float {
+      const int i0 = cnbasis(D, mode_degree(D, row));  // the first index of higher degree
+      const float* drow = sDm + (cc * NB1 + row) * NB4;
+      f2 s = f2_zero();
+#pragma unroll
+      for (int i = 0; i < NB; i += 4)
+        if (i + 4 > i0) {
+          f2 t[2];
+          lds_f2(drow + i, t[0], t[1]);
+#pragma unroll
+          for (int w = 0; w < 2; ++w)
+            if (i + 2 * w + 2 > i0 && i + 2 * w < NB) s = f2_fma(t[w], x[i / 2 + w < NP ? i / 2 + w : 0], s);
+        }
+      return f2_sum(s);
+    };
+    // separate wind: modal coefficients of div^ W = sum_a d^_a W_a, a term from each lane
+    f2 dw[WSEP ? NP1 : 1];
+    if constexpr (WSEP) {
+      float pd[NB1];
+#pragma unroll
+      for (int j = 0; j < NB1; ++j) pd[j] = derivative(cw, a, j);
+      __syncwarp();  // keeps the products of the two derivatives apart (registers)
+#pragma unroll
+      for (int j = 0; j < NB1; ++j) {
+        const float v = pd[j];
+        pd[j] += __shfl_sync(kFull, v, p1);
+        if (D == 3) pd[j] += __shfl_sync(kFull, v, p2);
+      }
+#pragma unroll
+      for (int j = 0; j < NP1; ++j) dw[j] = f2_pack(pd[2 * j], 2 * j + 1 < NB1 ? pd[2 * j + 1 < NB1 ? 2 * j + 1 : 0] : 0.0f);
+      __syncwarp();
+    }
+    // modal reference gradients of u_a (not with GTAB)
+    constexpr int NG1 = GTAB ? 1 : NP1;
+    f2 G[D][NG1];
     if constexpr (!GTAB) {
 #pragma unroll
       for (int cc = 0; cc < D; ++cc)
 #pragma unroll
-        for (int j = 0; j < NG1; ++j) {
-          const float* drow = sDm + (cc * NB1 + j) * NB4;
-          float p0 = 0.0f, p1s = 0.0f;
-#pragma unroll
-          for (int i = 0; i < NB; i += 4) {
-            float dv[4];
-            lds_v(drow + i, dv);
-#pragma unroll
-            for (int w = 0; w < 4; ++w)
-              if (i + w < NB) {
-                if (w & 1) p1s = fmaf(dv[w], c[i + w], p1s);
-                else p0 = fmaf(dv[w], c[i + w], p0);
-              }
-          }
-          G[cc][j] = p0 + p1s;
-        }
+        for (int j = 0; j < NP1; ++j)
+          G[cc][j] = f2_pack(derivative(c, cc, 2 * j), 2 * j + 1 < NB1 ? derivative(c, cc, 2 * j + 1) : 0.0f);
     }
-    float r[NB];
+    f2 r[NP];
 #pragma unroll
-    for (int i = 0; i < NB; ++i) r[i] = 0.0f;
-    // u_a and the reference gradient of u_a at point q
-    auto point_values = [&](int q, float& u, float (&gd)[D]) {
-      const float* ph = sBt + q * NBQ;
-      float u0 = 0.0f, u1 = 0.0f;
+    for (int j = 0; j < NP; ++j) r[j] = f2_zero();
+    // two points per pass where the registers allow it: the loads and shuffles of one overlap
+    // the arithmetic of the other (an odd last point is paired with itself at weight 0)
+    constexpr int XP = C::XP;
+    // Separate wind, many points: the test sums run in blocks of points whose partial sums meet
+    // in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
+    // more than the warp-per-element kernel, whose points are summed pairwise.
+    constexpr int QB = (WSEP && NQ > 64) ? (NQ / 8 + 1) * 2 : NQ;
+    float* yp = sY + ((act ? el : 0) * D + a) * NB;  // this lane's output entries
+#pragma unroll 1
+    for (int q0 = 0; q0 < NQ; q0 += QB) {
+      const int qe = q0 + QB < NQ ? q0 + QB : NQ;
+#pragma unroll 1
+      for (int q = q0; q < qe; q += XP) {
+        const bool two = q + 1 < NQ;
+        const int qs[2] = {q, two ? q + 1 : q};
+        float u[XP], gd[XP][D], wa[XP], dvs[XP];
+        {
+          f2 us[XP], gs[XP][D], ws[XP], ds[XP];
 #pragma unroll
-      for (int cc = 0; cc < D; ++cc) gd[cc] = 0.0f;
+          for (int x = 0; x < XP; ++x) {
+            us[x] = ws[x] = ds[x] = f2_zero();
 #pragma unroll
-      for (int i = 0; i < NB; i += 4) {
-        float pv[4];
-        lds_v(ph + i, pv);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const int idx = i + w;
-          if (idx < NB) {
-            if (w & 1) u1 = fmaf(pv[w], c[idx], u1);
-            else u0 = fmaf(pv[w], c[idx], u0);
+            for (int cc = 0; cc < D; ++cc) gs[x][cc] = f2_zero();
           }
-          if constexpr (!GTAB) {
-            if (idx < NB1) {
 #pragma unroll
-              for (int cc = 0; cc < D; ++cc) gd[cc] = fmaf(pv[w], G[cc][idx < NG1 ? idx : 0], gd[cc]);
+          for (int i = 0; i < NB; i += 4)
+#pragma unroll
+            for (int x = 0; x < XP; ++x) {
+              f2 t[2];
+              lds_f2(sBt + qs[x] * NBQ + i, t[0], t[1]);
+#pragma unroll
+              for (int w = 0; w < 2; ++w) {
+                const int j = i / 2 + w;
+                if (j < NP) us[x] = f2_fma(t[w], c[j < NP ? j : 0], us[x]);
+                if constexpr (WSEP) {
+                  if (j < NP) ws[x] = f2_fma(t[w], cw[j < NP ? j : 0], ws[x]);
+                  if (j < NP1) ds[x] = f2_fma(t[w], dw[j < NP1 ? j : 0], ds[x]);
+                }
+                if constexpr (!GTAB) {
+                  if (j < NP1) {
+#pragma unroll
+                    for (int cc = 0; cc < D; ++cc) gs[x][cc] = f2_fma(t[w], G[cc][j < NG1 ? j : 0], gs[x][cc]);
+                  }
+                }
+              }
+            }
+          if constexpr (GTAB) {  // d^_c u_a = sum_i (d phi_i / d xhat_c)(x_q) c_i
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc)
+#pragma unroll
+              for (int i = 0; i < NB; i += 4)
+#pragma unroll
+                for (int x = 0; x < XP; ++x) {
+                  f2 t[2];
+                  lds_f2(sm + C::O_DBT + (cc * NQ + qs[x]) * NBQ + i, t[0], t[1]);
+#pragma unroll
+                  for (int w = 0; w < 2; ++w)
+                    if (i / 2 + w < NP) gs[x][cc] = f2_fma(t[w], c[i / 2 + w < NP ? i / 2 + w : 0], gs[x][cc]);
+                }
+          }
+#pragma unroll
+          for (int x = 0; x < XP; ++x) {
+            u[x] = f2_sum(us[x]);
+            wa[x] = WSEP ? f2_sum(ws[x]) : u[x];
+            dvs[x] = f2_sum(ds[x]);
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) gd[x][cc] = f2_sum(gs[x][cc]);
+          }
+        }
+        f2 ff[XP];
+#pragma unroll
+        for (int x = 0; x < XP; ++x) {
+          float f;
+          if constexpr (WSEP) {
+            f = dvs[x] * u[x];
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) f = fmaf(__shfl_sync(kFull, wa[x], el * D + cc), gd[x][cc], f);
+          } else {
+            // W = M u with the other components' u; div^ W = sum_b sum_c M[c][b] d^_c u_b
+            const float u1 = __shfl_sync(kFull, u[x], p1);
+            const float u2 = D == 3 ? __shfl_sync(kFull, u[x], p2) : 0.0f;
+            float pd = 0.0f;
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) pd = fmaf(M0[cc], gd[x][cc], pd);
+            float dv = pd + __shfl_sync(kFull, pd, p1);
+            if (D == 3) dv += __shfl_sync(kFull, pd, p2);
+            f = dv * u[x];
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) {
+              float W = fmaf(M1[cc], u1, M0[cc] * u[x]);
+              if (D == 3) W = fmaf(M2[cc], u2, W);
+              f = fmaf(W, gd[x][cc], f);
             }
           }
+          ff[x] = f2_dup(f * (x == 0 || two ? sWq[qs[x]] : 0.0f));
+        }
+#pragma unroll
+        for (int i = 0; i < NB; i += 4) {
+          f2 t[XP][2];
+#pragma unroll
+          for (int x = 0; x < XP; ++x) lds_f2(sBt + qs[x] * NBQ + i, t[x][0], t[x][1]);
+#pragma unroll
+          for (int x = 0; x < XP; ++x)
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+              const int j = i / 2 + w;
+              if (j < NP) r[j < NP ? j : 0] = f2_fma(t[x][w], ff[x], r[j < NP ? j : 0]);
+            }
         }
       }
-      if constexpr (GTAB) {  // d^_c u_a = sum_i (d phi_i / d xhat_c)(x_q) c_i
+      if (QB < NQ && qe < NQ) {
 #pragma unroll
-        for (int cc = 0; cc < D; ++cc) {
-          const float* dph = sm + C::O_DBT + (cc * NQ + q) * NBQ;
-          float s0 = 0.0f, s1 = 0.0f;
-#pragma unroll
-          for (int i = 0; i < NB; i += 4) {
-            float pv[4];
-            lds_v(dph + i, pv);
-#pragma unroll
-            for (int w = 0; w < 4; ++w)
-              if (i + w < NB) {
-                if (w & 1) s1 = fmaf(pv[w], c[i + w], s1);
-                else s0 = fmaf(pv[w], c[i + w], s0);
-              }
+        for (int j = 0; j < NP; ++j) {
+          if (act) {
+            yp[2 * j] = f2_x(r[j]) + (q0 ? yp[2 * j] : 0.0f);
+            if (2 * j + 1 < NB) yp[2 * j + 1] = f2_y(r[j]) + (q0 ? yp[2 * j + 1] : 0.0f);
           }
-          gd[cc] = s0 + s1;
+          r[j] = f2_zero();
         }
-      }
-      u = u0 + u1;
-    };
-    // two points per pass: the loads and shuffles of one overlap the arithmetic of the other
-    // (an odd last point is paired with itself at weight 0)
-#pragma unroll 1
-    for (int q = 0; q < NQ; q += 2) {
-      const bool two = q + 1 < NQ;
-      const int qb = two ? q + 1 : q;
-      float ua, ub, ga[D], gb[D];
-      point_values(q, ua, ga);
-      point_values(qb, ub, gb);
-      float pda = 0.0f, pdb = 0.0f, pwa[D], pwb[D];
-#pragma unroll
-      for (int cc = 0; cc < D; ++cc) {
-        pda = fmaf(Mcol[cc], ga[cc], pda);
-        pdb = fmaf(Mcol[cc], gb[cc], pdb);
-        pwa[cc] = Mcol[cc] * ua;
-        pwb[cc] = Mcol[cc] * ub;
-      }
-      // sums over the element's D lanes: W_c = sum_b M[c][b] u_b, div^ W = sum_b sum_c M[c][b] d^_c u_b
-      float Wa[D], Wb[D];
-#pragma unroll
-      for (int cc = 0; cc < D; ++cc) {
-        Wa[cc] = pwa[cc] + __shfl_sync(kFull, pwa[cc], p1);
-        Wb[cc] = pwb[cc] + __shfl_sync(kFull, pwb[cc], p1);
-        if (D == 3) {
-          Wa[cc] += __shfl_sync(kFull, pwa[cc], p2);
-          Wb[cc] += __shfl_sync(kFull, pwb[cc], p2);
-        }
-      }
-      float dva = pda + __shfl_sync(kFull, pda, p1), dvb = pdb + __shfl_sync(kFull, pdb, p1);
-      if (D == 3) {
-        dva += __shfl_sync(kFull, pda, p2);
-        dvb += __shfl_sync(kFull, pdb, p2);
-      }
-      float fa = dva * ua, fb = dvb * ub;
-#pragma unroll
-      for (int cc = 0; cc < D; ++cc) {
-        fa = fmaf(Wa[cc], ga[cc], fa);
-        fb = fmaf(Wb[cc], gb[cc], fb);
-      }
-      fa *= sWq[q];
-      fb *= two ? sWq[qb] : 0.0f;
-      const float* pha = sBt + q * NBQ;
-      const float* phb = sBt + qb * NBQ;
-#pragma unroll
-      for (int i = 0; i < NB; i += 4) {
-        float va[4], vb[4];
-        lds_v(pha + i, va);
-        lds_v(phb + i, vb);
-#pragma unroll
-        for (int w = 0; w < 4; ++w)
-          if (i + w < NB) r[i + w] = fmaf(fb, vb[w], fmaf(fa, va[w], r[i + w]));
       }
     }
     // facet lift of component a: r_i += sum_fm TrM[fm][i] gam[e][fm][a]
     cp_wait<0>();
     __syncwarp();
     {
-      const float* gl = sG + el * NG + a;
-#pragma unroll 4
-      for (int fm = 0; fm < (D + 1) * NF; ++fm) {
-        const float gv = gl[fm * D];
-        const float* trow = sTrM + fm * NB4;
+      const float* gl = sG + (act ? el : 0) * NG + a;
+#pragma unroll 1
+      for (int f = 0; f <= D; ++f) {
 #pragma unroll
-        for (int i = 0; i < NB; i += 4) {
-          float tv[4];
-          lds_v(trow + i, tv);
+        for (int mm = 0; mm < NF; ++mm) {
+          const f2 gv = f2_dup(gl[(f * NF + mm) * D]);
+          const int i0 = cnbasis(D, mode_degree(D - 1, mm) - 1);  // lower degrees have no such trace
+          const float* trow = sTrM + (f * NF + mm) * NB4;
 #pragma unroll
-          for (int w = 0; w < 4; ++w)
-            if (i + w < NB) r[i + w] = fmaf(tv[w], gv, r[i + w]);
+          for (int i = 0; i < NB; i += 4)
+            if (i + 4 > i0) {
+              f2 t[2];
+              lds_f2(trow + i, t[0], t[1]);
+#pragma unroll
+              for (int w = 0; w < 2; ++w) {
+                const int j = i / 2 + w;
+                if (j < NP && 2 * j + 2 > i0) r[j < NP ? j : 0] = f2_fma(t[w], gv, r[j < NP ? j : 0]);
+              }
+            }
         }
+      }
+    }
+    if constexpr (QB < NQ) {
+      if (act) {
+#pragma unroll
+        for (int j = 0; j < NP; ++j) r[j] = f2_add(r[j], f2_pack(yp[2 * j], 2 * j + 1 < NB ? yp[2 * j + 1] : 0.0f));
       }
     }
     // inverse mass, then coalesced stores of the warp's element records
     if (act) {
 #pragma unroll
-      for (int i = 0; i < NB; ++i) sY[(el * D + a) * NB + i] = r[i] * invabs;
+      for (int j = 0; j < NP; ++j) {
+        yp[2 * j] = f2_x(r[j]) * invabs;
+        if (2 * j + 1 < NB) yp[2 * j + 1] = f2_y(r[j]) * invabs;
+      }
     }
     __syncwarp();
     if constexpr (!FUSE) {
@@ -294,31 +416,33 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB>::WARPS, VolR<D, K, GTAB>
       float Pi[D];
 #pragma unroll
       for (int cc = 0; cc < D; ++cc) Pi[cc] = float(__ldg(gp + D * D + a * D + cc));
+      const float* ye = sY + (act ? el : 0) * NL;
 #pragma unroll
-      for (int i = 0; i < NB; ++i) {
-        float acc = 0.0f;
+      for (int j = 0; j < NP; ++j) {
+        float v[2] = {0.0f, 0.0f};
 #pragma unroll
-        for (int cc = 0; cc < D; ++cc) acc = fmaf(Pi[cc], sY[el * NL + cc * NB + i], acc);
-        r[i] = acc;
+        for (int w = 0; w < 2; ++w)
+          if (2 * j + w < NB) {
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) v[w] = fmaf(Pi[cc], ye[cc * NB + 2 * j + w], v[w]);
+          }
+        r[j] = f2_pack(v[0], v[1]);
       }
       const float* sD = sm + C::O_D + a * NB4;
       const int* codes = m.efc + e * (D + 1);
 #pragma unroll 1
       for (int rr = 0; rr < NL; ++rr) {
         const float* drow = sD + rr * C::NDP;
-        float p0 = 0.0f, p1s = 0.0f;
+        f2 s = f2_zero();
 #pragma unroll
         for (int i = 0; i < NB; i += 4) {
-          float dv[4];
-          lds_v(drow + i, dv);
+          f2 t[2];
+          lds_f2(drow + i, t[0], t[1]);
 #pragma unroll
-          for (int w = 0; w < 4; ++w)
-            if (i + w < NB) {
-              if (w & 1) p1s = fmaf(dv[w], r[i + w], p1s);
-              else p0 = fmaf(dv[w], r[i + w], p0);
-            }
+          for (int w = 0; w < 2; ++w)
+            if (i / 2 + w < NP) s = f2_fma(t[w], r[i / 2 + w < NP ? i / 2 + w : 0], s);
         }
-        const float part = p0 + p1s;
+        const float part = f2_sum(s);
         float v = part + __shfl_sync(kFull, part, p1);
         if (D == 3) v += __shfl_sync(kFull, part, p2);
         if (act && rr / NB == a) {

@@ -1,31 +1,38 @@
-// a3 + a5 with the element's data in registers, the basis split over two lanes (FP32,
-// STAGE wind w = u): volume term, facet lift and inverse mass.
+// a3 + a5 with the element's data in registers, the basis split over two lanes (FP32): volume
+// term, facet lift and inverse mass.
 //
 // The structure of k_volume_r (a lane per (element, component a), the quadrature points
-// walked in the same order by every lane, broadcast basis rows, W and div^ W summed over
-// the element's lanes by shuffles, f_a = w_q (div^W u_a + W . grad^ u_a) tested against
-// phi_i), with each (element, component) pair on two lanes: half h owns the basis indices
-// i = 2 t + h (coefficients c_i, test accumulators r_i) and the modal gradient entries
-// G_c[j], j = 2 t + h < dim P^{k-1}.  Per point a lane forms its half's partial sums of u_a
-// and d^_c u_a, and one shuffle with the other half completes them; both halves then hold
-// the same f_a and accumulate their own r_i.  The tables are staged with their basis columns
-// permuted so that each half reads one contiguous block of a row (half h at column offset
-// h HP).  Half the registers per lane of k_volume_r: twice the resident warps at k = 4, and
-// a register kernel at all at k = 5 (where a whole basis does not fit in one lane).
+// walked in the same order by every lane, broadcast basis rows, the other components taken
+// by shuffles, f_a = w_q (div^W u_a + W . grad^ u_a) tested against phi_i, register pairs, the
+// products that vanish by degree left out), with each (element, component) pair on two
+// lanes: half h owns the basis indices i = 2 t + h (coefficients c_i, test accumulators r_i,
+// with a separate wind its coefficients) and the modal gradient entries G_c[j], j = 2 t + h <
+// dim P^{k-1} (and those of div^ W).  Per point a lane forms its half's partial sums, and one
+// shuffle each with the other half completes them; both halves then hold the same f_a and
+// accumulate their own r_i.  The tables are staged with their basis columns permuted so that
+// each half reads one contiguous block of a row (half h at column offset h HP).  Half the
+// registers per lane of k_volume_r: a register kernel at k = 5, where a whole basis does not
+// fit in one lane.  WSEP: a wind of its own, as in k_volume_r.
+//
+// Bound: FMA register reads and the shuffles.  Measured (CUDA events, per launch): 18^3 x 6,
+// k = 5, w = u 437 -> 351 us (scalar FMAs, dense Dm and TrM products before); 13^3 x 6, k = 5,
+// separate wind 633 -> 192 us (a warp per element before).
 #pragma once
+#include "f32x2.cuh"
 #include "kernels.cuh"
+#include "kernels_vr.cuh"
 
 namespace hopu {
 
-template <int D, int K>
+template <int D, int K, bool WSEP = false>
 struct VolRH {
   using S = Shape<D, K>;
   static constexpr int NB = S::nb, NB1 = cnbasis(D, K - 1), NF = S::nf, NL = S::nloc, NQ = S::nq, GT = S::gt;
   static constexpr int LPE = 2 * D;               // lanes per element: (component, half)
   static constexpr int ELW = 32 / LPE;            // elements per warp
-  static constexpr int WARPS = 8;
   static constexpr int NH = (NB + 1) / 2;         // basis indices of half 0 (half 1: NB - NH)
   static constexpr int NH1 = (NB1 + 1) / 2;       // modal-gradient indices of half 0
+  static constexpr int NP = (NH + 1) / 2, NP1 = (NH1 + 1) / 2;  // pairs of a half
   static constexpr int HP = r4i(NH);              // one half's block of a permuted row
   static constexpr int RW = 2 * HP;               // permuted row width
   static constexpr int NBQ = (RW / 4) % 2 == 0 ? RW + 4 : RW;  // Bt row stride: an odd multiple of 16 bytes
@@ -34,25 +41,26 @@ struct VolRH {
   static constexpr int O_DM = r4i(O_WQ + NQ);     // Dm [D][NB1][RW], permuted columns
   static constexpr int O_TRM = O_DM + D * NB1 * RW;   // TrM [(D+1) NF][RW], permuted columns
   static constexpr int O_W = O_TRM + (D + 1) * NF * RW;
-  static constexpr int PER_WARP = r4i(ELW * NL);  // output staging of the warp's elements
-  static constexpr int GW = r4i(ELW * NG);        // the warp's facet moments, staged by cp.async
-  static constexpr int O_G = O_W + WARPS * PER_WARP;
+  static constexpr int PER_WARP = r4i(ELW * NL);  // the warp's element records: in (u, w), and out
+  static constexpr int GW = r4i(ELW * NG);        // the warp's facet moments
+  static constexpr int NBUF = WSEP ? 3 : 2;
+  // tables above 64 KB: one CTA of 8 warps per SM; else CTAs of 4 warps, as many as fit
+  static constexpr int WARPS = O_W * 4 > 64 * 1024 ? 8 : 4;
+  static constexpr int O_G = O_W + WARPS * NBUF * PER_WARP;
   static constexpr size_t SMEM = size_t(O_G + WARPS * GW) * 4;
-  static constexpr int REGS = 2 * NH + D * NH1;   // c, r and G of a lane
-  static constexpr int MINB = 2 * SMEM <= 200 * 1024 ? 2 : 1;
-  static constexpr bool OK = REGS <= 128 && SMEM <= 200 * 1024 && NB >= 2;
-  // permuted column of basis index i
-  static constexpr __host__ __device__ int col(int i) { return (i & 1) * HP + (i >> 1); }
+  static constexpr int REGS = (WSEP ? 3 * NH + NH1 : 2 * NH) + D * NH1;  // a lane's vectors
+  static constexpr int MINB = WARPS == 8 ? 1 : (REGS <= 60 ? 4 : 3);
+  static constexpr bool OK = REGS <= 160 && SMEM <= 220 * 1024 && NB >= 2;
 };
 
-template <int D, int K>
-__global__ void __launch_bounds__(32 * VolRH<D, K>::WARPS, VolRH<D, K>::MINB)
-    k_volume_rh(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ gam, float* out,
-                Combine cmb) {
-  using C = VolRH<D, K>;
+template <int D, int K, bool WSEP>
+__global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSEP>::MINB)
+    k_volume_rh(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ wL,
+                const float* __restrict__ gam, float* out, Combine cmb) {
+  using C = VolRH<D, K, WSEP>;
   constexpr int NB = C::NB, NB1 = C::NB1, NF = C::NF, NL = C::NL, NQ = C::NQ, GT = C::GT;
   constexpr int NBQ = C::NBQ, HP = C::HP, RW = C::RW, NG = C::NG, ELW = C::ELW, LPE = C::LPE;
-  constexpr int NH = C::NH, NH1 = C::NH1;
+  constexpr int NH = C::NH, NH1 = C::NH1, NP = C::NP, NP1 = C::NP1;
   extern __shared__ __align__(16) float sm[];
   pdl_trigger();
   {  // tables with permuted basis columns (zero padding)
@@ -86,174 +94,266 @@ __global__ void __launch_bounds__(32 * VolRH<D, K>::WARPS, VolRH<D, K>::MINB)
   const int el = lane_on ? lane / LPE : 0;
   const int rr = lane_on ? lane - el * LPE : 0;
   const int a = rr >> 1, h = rr & 1;
+  const int a1 = (a + 1) % D, a2 = (a + 2) % D;
   const int nh = h ? NB - NH : NH;          // this half's basis indices
-  const int nh1 = h ? NB1 - NH1 : NH1;      // and modal-gradient indices
   const int pt = lane ^ 1;                  // the other half of this (element, component)
   // the other components' lanes of the same half (idle lanes talk to themselves)
-  const int p1 = lane_on ? el * LPE + ((a + 1) % D) * 2 + h : lane;
-  const int p2 = lane_on ? el * LPE + ((a + 2) % D) * 2 + h : lane;
-  float* sY = sm + C::O_W + warp * C::PER_WARP;
+  const int p1 = lane_on ? el * LPE + a1 * 2 + h : lane;
+  const int p2 = lane_on ? el * LPE + a2 * 2 + h : lane;
+  float* sIn = sm + C::O_W + warp * C::NBUF * C::PER_WARP;
+  float* sY = sIn + C::PER_WARP;
+  float* sWn = sY + (WSEP ? C::PER_WARP : 0);
   float* sG = sm + C::O_G + warp * C::GW;
-  const int64_t ngroups = (m.E + ELW - 1) / ELW;
-  for (int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x; grp < ngroups; grp += (int64_t)gridDim.x * C::WARPS) {
+  const int64_t ngroups = (m.E + ELW - 1) / ELW, gstep = (int64_t)gridDim.x * C::WARPS;
+  auto count = [&](int64_t g) { return (m.E - g * ELW < ELW) ? (int)(m.E - g * ELW) : ELW; };
+  auto request = [&](int64_t g) {
+    warp_copy_records<NL, ELW>(sIn, uL, g * ELW, count(g), lane);
+    if (WSEP) warp_copy_records<NL, ELW>(sWn, wL, g * ELW, count(g), lane);
+  };
+  auto halves = [&](float v) { return v + __shfl_sync(kFull, v, pt); };
+  int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x;
+  if (grp < ngroups) request(grp);
+  cp_commit();
+  for (; grp < ngroups; grp += gstep) {
     const int64_t e0 = grp * ELW;
-    const int ne = (m.E - e0 < ELW) ? (int)(m.E - e0) : ELW;
+    const int ne = count(grp);
     const bool act = lane_on && el < ne;
     const int64_t e = act ? e0 + el : e0;  // inactive lanes read the group's first element
-    // the group's facet moments arrive in shared memory while the points are walked
-    for (int k2 = 0; k2 < ne; ++k2) warp_copy_async<NG * 4>(sG + k2 * NG, gam + (e0 + k2) * NG, lane);
-    cp_commit();
-    // this half's coefficients c[t] = c_a[2 t + h] (zero beyond the half)
-    float c[NH];
-    {
-      const float* up = uL + e * NL + a * NB + h;
-#pragma unroll
-      for (int t = 0; t < NH; ++t) c[t] = (t < nh) ? __ldg(up + 2 * t) : 0.0f;
-    }
     const double* gp = m.geoT + e * GT;
-    float Mcol[D];  // column a of M = |det J| J^-1
+    // M = |det J| J^-1: its columns a, a + 1, a + 2 (w = u), or its row a in M0 (separate wind)
+    float M0[D], M1[WSEP ? 1 : D], M2[WSEP ? 1 : D];
 #pragma unroll
-    for (int cc = 0; cc < D; ++cc) Mcol[cc] = float(__ldg(gp + 2 * D * D + cc * D + a));
+    for (int cc = 0; cc < D; ++cc) {
+      M0[cc] = float(__ldg(gp + 2 * D * D + (WSEP ? a * D + cc : cc * D + a)));
+      if constexpr (!WSEP) {
+        M1[cc] = float(__ldg(gp + 2 * D * D + cc * D + a1));
+        M2[cc] = D == 3 ? float(__ldg(gp + 2 * D * D + cc * D + a2)) : 0.0f;
+      }
+    }
     const float invabs = float(__ldg(gp + 3 * D * D));
-    // this half's modal gradient entries G[cc][t1] = sum_i Dm[cc][2 t1 + h][i] c_i, with the
-    // other half's coefficients taken once from the partner lane
-    float G[D][NH1];
+    // this half's coefficients, c_a[2 t + h] (zero beyond the half)
+    f2 c[NP], cw[WSEP ? NP : 1];
+    cp_wait<0>();
+    __syncwarp();
     {
-      float co[NH];
+      const int o = ((act ? el : 0) * D + a) * NB + h;
 #pragma unroll
-      for (int t = 0; t < NH; ++t) co[t] = __shfl_sync(kFull, c[t], pt);
+      for (int j = 0; j < NP; ++j) {
+        const bool in0 = 2 * j < nh, in1 = 2 * j + 1 < nh;
+        c[j] = f2_pack(in0 ? sIn[o + 4 * j] : 0.0f, in1 ? sIn[o + 4 * j + 2] : 0.0f);
+        if constexpr (WSEP) {  // modal W_a = sum_b M[a][b] w_b, the wind's reference component a
+          float v[2] = {0.0f, 0.0f};
+          const float* wp = sWn + (act ? el : 0) * NL + h + 4 * j;
+#pragma unroll
+          for (int b = 0; b < D; ++b) {
+            if (in0) v[0] = fmaf(M0[b], wp[b * NB], v[0]);
+            if (in1) v[1] = fmaf(M0[b], wp[b * NB + 2], v[1]);
+          }
+          cw[j] = f2_pack(v[0], v[1]);
+        }
+      }
+    }
+    __syncwarp();
+    // this group's facet moments and the next group's coefficients arrive during the points
+    warp_copy_records<NG, ELW>(sG, gam, e0, ne, lane);
+    if (grp + gstep < ngroups) request(grp + gstep);
+    cp_commit();
+    // this half's entry j = 2 t + h of the modal reference derivative sum_i Dm[cc][j][i] x_i, xo
+    // the other half's coefficients (zero past dim P^{k-1})
+    auto derivative = [&](const f2 (&x)[NP], const f2 (&xo)[NP], int cc, int t) -> float {
+      const int j = 2 * t + h;
+      const bool in = j < NB1;
+      const int i0 = cnbasis(D, mode_degree(D, 2 * t));  // no terms below: the lower of the two halves' rows
+      const float* drow = sDm + (cc * NB1 + (in ? j : 0)) * RW;
+      const float* mine = drow + h * HP;
+      const float* other = drow + (1 - h) * HP;
+      f2 s0 = f2_zero(), s1 = f2_zero();
+#pragma unroll
+      for (int t4 = 0; t4 < NH; t4 += 4)
+        if (2 * t4 + 8 > i0) {
+          f2 d[2], o[2];
+          lds_f2(mine + t4, d[0], d[1]);
+          lds_f2(other + t4, o[0], o[1]);
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            const int jj = t4 / 2 + w;
+            if (jj < NP && 4 * jj + 4 > i0) {
+              s0 = f2_fma(d[w], x[jj < NP ? jj : 0], s0);
+              s1 = f2_fma(o[w], xo[jj < NP ? jj : 0], s1);
+            }
+          }
+        }
+      return in ? f2_sum(f2_add(s0, s1)) : 0.0f;
+    };
+    auto swap = [&](const f2 (&x)[NP], f2 (&xo)[NP]) {
+#pragma unroll
+      for (int j = 0; j < NP; ++j)
+        xo[j] = f2_pack(__shfl_sync(kFull, f2_x(x[j]), pt), __shfl_sync(kFull, f2_y(x[j]), pt));
+    };
+    // separate wind: this half's modal coefficients of div^ W = sum_a d^_a W_a, a term per lane
+    f2 dw[WSEP ? NP1 : 1];
+    if constexpr (WSEP) {
+      f2 xo[NP];
+      swap(cw, xo);
+      float pd[2 * NP1];
+#pragma unroll
+      for (int t = 0; t < 2 * NP1; ++t) pd[t] = t < NH1 ? derivative(cw, xo, a, t) : 0.0f;
+      __syncwarp();  // keeps the products of the two derivatives apart (registers)
+#pragma unroll
+      for (int t = 0; t < NH1; ++t) {
+        const float v = pd[t];
+        pd[t] += __shfl_sync(kFull, v, p1);
+        if (D == 3) pd[t] += __shfl_sync(kFull, v, p2);
+      }
+#pragma unroll
+      for (int j = 0; j < NP1; ++j) dw[j] = f2_pack(pd[2 * j], pd[2 * j + 1]);
+      __syncwarp();
+    }
+    // modal reference gradients of u_a
+    f2 G[D][NP1];
+    {
+      f2 xo[NP];
+      swap(c, xo);
 #pragma unroll
       for (int cc = 0; cc < D; ++cc)
 #pragma unroll
-        for (int t1 = 0; t1 < NH1; ++t1) {
-          const int j = 2 * t1 + h;
-          const float* drow = sDm + (cc * NB1 + (j < NB1 ? j : 0)) * RW;
-          const float* mine = drow + h * HP;
-          const float* other = drow + (1 - h) * HP;
-          float s0 = 0.0f, s1 = 0.0f;
-#pragma unroll
-          for (int t = 0; t < NH; t += 4) {
-            float dv[4], ov[4];
-            lds_v(mine + t, dv);
-            lds_v(other + t, ov);
-#pragma unroll
-            for (int w = 0; w < 4; ++w)
-              if (t + w < NH) {
-                s0 = fmaf(dv[w], c[t + w], s0);
-                s1 = fmaf(ov[w], co[t + w], s1);
-              }
-          }
-          G[cc][t1] = (t1 < nh1) ? s0 + s1 : 0.0f;
-        }
+        for (int j = 0; j < NP1; ++j)
+          G[cc][j] = f2_pack(derivative(c, xo, cc, 2 * j), 2 * j + 1 < NH1 ? derivative(c, xo, cc, 2 * j + 1) : 0.0f);
     }
-    float r[NH];
+    f2 r[NP];
 #pragma unroll
-    for (int t = 0; t < NH; ++t) r[t] = 0.0f;
-    // u_a and the reference gradient of u_a at point q: this half's partial sums, completed
-    // by one shuffle each with the other half
-    auto point_values = [&](int q, float& u, float (&gd)[D]) {
-      const float* ph = sBt + q * NBQ + h * HP;
-      float u0 = 0.0f, u1 = 0.0f;
-#pragma unroll
-      for (int cc = 0; cc < D; ++cc) gd[cc] = 0.0f;
-#pragma unroll
-      for (int t = 0; t < NH; t += 4) {
-        float pv[4];
-        lds_v(ph + t, pv);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const int idx = t + w;
-          if (idx < NH) {
-            if (w & 1) u1 = fmaf(pv[w], c[idx], u1);
-            else u0 = fmaf(pv[w], c[idx], u0);
-          }
-          if (idx < NH1) {
-#pragma unroll
-            for (int cc = 0; cc < D; ++cc) gd[cc] = fmaf(pv[w], G[cc][idx < NH1 ? idx : 0], gd[cc]);
-          }
-        }
-      }
-      const float up = u0 + u1;
-      u = up + __shfl_sync(kFull, up, pt);
-#pragma unroll
-      for (int cc = 0; cc < D; ++cc) gd[cc] += __shfl_sync(kFull, gd[cc], pt);
-    };
+    for (int j = 0; j < NP; ++j) r[j] = f2_zero();
     // two points per pass (an odd last point is paired with itself at weight 0)
+    // Separate wind, many points: the test sums run in blocks of points whose partial sums meet
+    // in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
+    // more than the warp-per-element kernel, whose points are summed pairwise.
+    constexpr int QB = (WSEP && NQ > 64) ? (NQ / 8 + 1) * 2 : NQ;
+    float* yp = sY + ((act ? el : 0) * D + a) * NB + h;  // this lane's output entries
 #pragma unroll 1
-    for (int q = 0; q < NQ; q += 2) {
-      const bool two = q + 1 < NQ;
-      const int qb = two ? q + 1 : q;
-      float ua, ub, ga[D], gb[D];
-      point_values(q, ua, ga);
-      point_values(qb, ub, gb);
-      float pda = 0.0f, pdb = 0.0f, pwa[D], pwb[D];
+    for (int q0 = 0; q0 < NQ; q0 += QB) {
+      const int qe = q0 + QB < NQ ? q0 + QB : NQ;
+#pragma unroll 1
+      for (int q = q0; q < qe; q += 2) {
+        const bool two = q + 1 < NQ;
+        const int qs[2] = {q, two ? q + 1 : q};
+        f2 us[2], gs[2][D], ws[2], ds[2], ff[2];
 #pragma unroll
-      for (int cc = 0; cc < D; ++cc) {
-        pda = fmaf(Mcol[cc], ga[cc], pda);
-        pdb = fmaf(Mcol[cc], gb[cc], pdb);
-        pwa[cc] = Mcol[cc] * ua;
-        pwb[cc] = Mcol[cc] * ub;
-      }
-      // sums over the element's components (lanes of the same half): W_c and div^ W
-      float Wa[D], Wb[D];
+        for (int x = 0; x < 2; ++x) {
+          us[x] = ws[x] = ds[x] = f2_zero();
 #pragma unroll
-      for (int cc = 0; cc < D; ++cc) {
-        Wa[cc] = pwa[cc] + __shfl_sync(kFull, pwa[cc], p1);
-        Wb[cc] = pwb[cc] + __shfl_sync(kFull, pwb[cc], p1);
-        if (D == 3) {
-          Wa[cc] += __shfl_sync(kFull, pwa[cc], p2);
-          Wb[cc] += __shfl_sync(kFull, pwb[cc], p2);
+          for (int cc = 0; cc < D; ++cc) gs[x][cc] = f2_zero();
+        }
+#pragma unroll
+        for (int t4 = 0; t4 < NH; t4 += 4)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            f2 p[2];
+            lds_f2(sBt + qs[x] * NBQ + h * HP + t4, p[0], p[1]);
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+              const int j = t4 / 2 + w, jc = j < NP ? j : 0, j1 = j < NP1 ? j : 0;
+              if (j < NP) us[x] = f2_fma(p[w], c[jc], us[x]);
+              if constexpr (WSEP) {
+                if (j < NP) ws[x] = f2_fma(p[w], cw[jc], ws[x]);
+                if (j < NP1) ds[x] = f2_fma(p[w], dw[j1], ds[x]);
+              }
+              if (j < NP1) {
+#pragma unroll
+                for (int cc = 0; cc < D; ++cc) gs[x][cc] = f2_fma(p[w], G[cc][j1], gs[x][cc]);
+              }
+            }
+          }
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const float u = halves(f2_sum(us[x]));
+          float gd[D];
+#pragma unroll
+          for (int cc = 0; cc < D; ++cc) gd[cc] = halves(f2_sum(gs[x][cc]));
+          float f;
+          if constexpr (WSEP) {
+            const float wa = halves(f2_sum(ws[x]));
+            f = halves(f2_sum(ds[x])) * u;
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) f = fmaf(__shfl_sync(kFull, wa, el * LPE + 2 * cc), gd[cc], f);
+          } else {
+            const float u1 = __shfl_sync(kFull, u, p1);
+            const float u2 = D == 3 ? __shfl_sync(kFull, u, p2) : 0.0f;
+            float pd = 0.0f;
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) pd = fmaf(M0[cc], gd[cc], pd);
+            float dv = pd + __shfl_sync(kFull, pd, p1);
+            if (D == 3) dv += __shfl_sync(kFull, pd, p2);
+            f = dv * u;
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) {
+              float W = fmaf(M1[cc], u1, M0[cc] * u);
+              if (D == 3) W = fmaf(M2[cc], u2, W);
+              f = fmaf(W, gd[cc], f);
+            }
+          }
+          ff[x] = f2_dup(f * (x == 0 || two ? sWq[qs[x]] : 0.0f));
+        }
+#pragma unroll
+        for (int t4 = 0; t4 < NH; t4 += 4) {
+          f2 ta[2], tc[2];
+          lds_f2(sBt + qs[0] * NBQ + h * HP + t4, ta[0], ta[1]);
+          lds_f2(sBt + qs[1] * NBQ + h * HP + t4, tc[0], tc[1]);
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            const int j = t4 / 2 + w;
+            if (j < NP) r[j < NP ? j : 0] = f2_fma(tc[w], ff[1], f2_fma(ta[w], ff[0], r[j < NP ? j : 0]));
+          }
         }
       }
-      float dva = pda + __shfl_sync(kFull, pda, p1), dvb = pdb + __shfl_sync(kFull, pdb, p1);
-      if (D == 3) {
-        dva += __shfl_sync(kFull, pda, p2);
-        dvb += __shfl_sync(kFull, pdb, p2);
-      }
-      float fa = dva * ua, fb = dvb * ub;
+      if (QB < NQ && qe < NQ) {
 #pragma unroll
-      for (int cc = 0; cc < D; ++cc) {
-        fa = fmaf(Wa[cc], ga[cc], fa);
-        fb = fmaf(Wb[cc], gb[cc], fb);
-      }
-      fa *= sWq[q];
-      fb *= two ? sWq[qb] : 0.0f;
-      const float* pha = sBt + q * NBQ + h * HP;
-      const float* phb = sBt + qb * NBQ + h * HP;
-#pragma unroll
-      for (int t = 0; t < NH; t += 4) {
-        float va[4], vb[4];
-        lds_v(pha + t, va);
-        lds_v(phb + t, vb);
-#pragma unroll
-        for (int w = 0; w < 4; ++w)
-          if (t + w < NH) r[t + w] = fmaf(fb, vb[w], fmaf(fa, va[w], r[t + w]));
+        for (int j = 0; j < NP; ++j) {
+          if (act && 2 * j < nh) yp[4 * j] = f2_x(r[j]) + (q0 ? yp[4 * j] : 0.0f);
+          if (act && 2 * j + 1 < nh) yp[4 * j + 2] = f2_y(r[j]) + (q0 ? yp[4 * j + 2] : 0.0f);
+          r[j] = f2_zero();
+        }
       }
     }
     // facet lift of component a, this half: r_t += sum_fm TrM[fm][2 t + h] gam[e][fm][a]
     cp_wait<0>();
     __syncwarp();
     {
-      const float* gl = sG + el * NG + a;
-#pragma unroll 4
-      for (int fm = 0; fm < (D + 1) * NF; ++fm) {
-        const float gv = gl[fm * D];
-        const float* trow = sTrM + fm * RW + h * HP;
+      const float* gl = sG + (act ? el : 0) * NG + a;
+#pragma unroll 1
+      for (int f = 0; f <= D; ++f) {
 #pragma unroll
-        for (int t = 0; t < NH; t += 4) {
-          float tv[4];
-          lds_v(trow + t, tv);
+        for (int mm = 0; mm < NF; ++mm) {
+          const f2 gv = f2_dup(gl[(f * NF + mm) * D]);
+          const int i0 = cnbasis(D, mode_degree(D - 1, mm) - 1);  // lower degrees have no such trace
+          const float* trow = sTrM + (f * NF + mm) * RW + h * HP;
 #pragma unroll
-          for (int w = 0; w < 4; ++w)
-            if (t + w < NH) r[t + w] = fmaf(tv[w], gv, r[t + w]);
+          for (int t4 = 0; t4 < NH; t4 += 4)
+            if (2 * t4 + 8 > i0) {
+              f2 t[2];
+              lds_f2(trow + t4, t[0], t[1]);
+#pragma unroll
+              for (int w = 0; w < 2; ++w) {
+                const int j = t4 / 2 + w;
+                if (j < NP && 4 * j + 4 > i0) r[j < NP ? j : 0] = f2_fma(t[w], gv, r[j < NP ? j : 0]);
+              }
+            }
         }
+      }
+    }
+    if constexpr (QB < NQ) {
+      if (act) {
+#pragma unroll
+        for (int j = 0; j < NP; ++j)
+          r[j] = f2_add(r[j], f2_pack(2 * j < nh ? yp[4 * j] : 0.0f, 2 * j + 1 < nh ? yp[4 * j + 2] : 0.0f));
       }
     }
     // inverse mass, then coalesced stores of the warp's element records
     if (act) {
 #pragma unroll
-      for (int t = 0; t < NH; ++t)
-        if (t < nh) sY[(el * D + a) * NB + 2 * t + h] = r[t] * invabs;
+      for (int j = 0; j < NP; ++j) {
+        if (2 * j < nh) yp[4 * j] = f2_x(r[j]) * invabs;
+        if (2 * j + 1 < nh) yp[4 * j + 2] = f2_y(r[j]) * invabs;
+      }
     }
     __syncwarp();
     for (int t = lane; t < ne * NL; t += 32) {

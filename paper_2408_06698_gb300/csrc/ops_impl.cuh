@@ -93,9 +93,14 @@ class OpsImpl final : public Ops {
   static constexpr bool kVolRF = std::is_same<T, float>::value && VolR<D, K>::FUSE_OK;
   static constexpr bool kVolRT = std::is_same<T, float>::value && VolR<D, K, true>::OK;
   int g_volrt_ = 1;
-  // register kernel with the basis split over two lanes
+  // register kernel with the basis split over two lanes; every FP32 order has one of the two
   static constexpr bool kVolRH = std::is_same<T, float>::value && VolRH<D, K>::OK;
+  static_assert(!std::is_same<T, float>::value || kVolR || kVolRH, "a register volume kernel for every FP32 order");
   int g_volrh_ = 1;
+  // separate wind in FP32: the register kernel, its half-basis form where a lane's registers run out
+  static constexpr bool kVolRW = std::is_same<T, float>::value && VolR<D, K, false, true>::OK;
+  static constexpr bool kVolRHW = std::is_same<T, float>::value && !kVolRW;
+  int g_volw_ = 1;
   // register-resident adjoint volume kernel (w = u)
   static constexpr bool kVolAR = std::is_same<T, float>::value && VolAR<D, K>::OK;
   int g_volar_ = 1;
@@ -239,10 +244,12 @@ class OpsImpl final : public Ops {
       if ((err = setup(k_facet<D, K, T, false, kFacetTab>, facet_smem(false), th, &g_fac_[0])) != cudaSuccess) return err;
       if ((err = setup(k_facet<D, K, T, true, kFacetTab>, facet_smem(true), th, &g_fac_[1])) != cudaSuccess) return err;
     }
-    if ((err = setup(k_volume<D, K, T, false, kVolumeTab, false>, volume_smem(false), th, &g_vol_[0])) != cudaSuccess) return err;
+    if constexpr (!std::is_same<T, float>::value) {
+      if ((err = setup(k_volume<D, K, T, false, kVolumeTab, false>, volume_smem(false), th, &g_vol_[0])) != cudaSuccess) return err;
+    }
     if ((err = setup(k_volume<D, K, T, true, kVolumeTab, false>, volume_smem(true), th, &g_vol_[1])) != cudaSuccess) return err;
     if constexpr (kVolR) {
-      if ((err = setup(k_volume_r<D, K, false, false>, VolR<D, K>::SMEM, 32 * VolR<D, K>::WARPS, &g_volr_)) != cudaSuccess)
+      if ((err = setup(k_volume_r<D, K, false, false, false>, VolR<D, K>::SMEM, 32 * VolR<D, K>::WARPS, &g_volr_)) != cudaSuccess)
         return err;
     }
     if constexpr (kFacAR) {
@@ -254,16 +261,24 @@ class OpsImpl final : public Ops {
         return err;
     }
     if constexpr (kVolRH) {
-      if ((err = setup(k_volume_rh<D, K>, VolRH<D, K>::SMEM, 32 * VolRH<D, K>::WARPS, &g_volrh_)) != cudaSuccess)
+      if ((err = setup(k_volume_rh<D, K, false>, VolRH<D, K>::SMEM, 32 * VolRH<D, K>::WARPS, &g_volrh_)) != cudaSuccess)
         return err;
     }
+    if constexpr (kVolRW) {
+      using R = VolR<D, K, false, true>;
+      if ((err = setup(k_volume_r<D, K, false, false, true>, R::SMEM, 32 * R::WARPS, &g_volw_)) != cudaSuccess) return err;
+    }
+    if constexpr (kVolRHW) {
+      using R = VolRH<D, K, true>;
+      if ((err = setup(k_volume_rh<D, K, true>, R::SMEM, 32 * R::WARPS, &g_volw_)) != cudaSuccess) return err;
+    }
     if constexpr (kVolRT) {
-      if ((err = setup(k_volume_r<D, K, false, true>, VolR<D, K, true>::SMEM, 32 * VolR<D, K, true>::WARPS,
+      if ((err = setup(k_volume_r<D, K, false, true, false>, VolR<D, K, true>::SMEM, 32 * VolR<D, K, true>::WARPS,
                        &g_volrt_)) != cudaSuccess)
         return err;
     }
     if constexpr (kVolRF) {
-      if ((err = setup(k_volume_r<D, K, true, false>, VolR<D, K>::SMEM_FUSE, 32 * VolR<D, K>::WARPS, &g_volrf_)) !=
+      if ((err = setup(k_volume_r<D, K, true, false, false>, VolR<D, K>::SMEM_FUSE, 32 * VolR<D, K>::WARPS, &g_volrf_)) !=
           cudaSuccess)
         return err;
     }
@@ -365,8 +380,8 @@ class OpsImpl final : public Ops {
       if (!wsep && (vvar_ == kVolRegHalf || !kVolR)) {
         using R = VolRH<D, K>;
         const int g = clamp_grid(g_volrh_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_rh<D, K>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(gam), static_cast<float*>(out), c);
+        launch(k_volume_rh<D, K, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(out), c);
         return 1;
       }
     }
@@ -374,8 +389,8 @@ class OpsImpl final : public Ops {
       if (!wsep && vvar_ == kVolRegTab) {
         using R = VolR<D, K, true>;
         const int g = clamp_grid(g_volrt_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_r<D, K, false, true>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
+        launch(k_volume_r<D, K, false, true, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
         return 1;
       }
     }
@@ -383,20 +398,44 @@ class OpsImpl final : public Ops {
       if (!wsep) {
         using R = VolR<D, K>;
         const int g = clamp_grid(g_volr_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_r<D, K, false, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
+        launch(k_volume_r<D, K, false, false, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
         return 1;
       }
     }
+    // Separate wind (and FP64).  FP32: the register kernels, except while the warp-per-element
+    // kernel has a resident warp for every element: its one pass is then shorter than a register
+    // warp's walk over 32 / D elements (FP32 k = 3, 162 elements: 10 against 16 us; 7986 elements:
+    // 27 against 20 us; k = 4, 2058 elements: 37 against 39 us; 6000 elements: 70 against 53 us).
     const int g = clamp_grid(g_vol_[wsep ? 1 : 0], m.E, kWarps);
-    if (wsep)
-      launch(k_volume<D, K, T, true, kVolumeTab, false>, g, 32 * kWarps, volume_smem(true), st, 
+    if constexpr (kVolRW || kVolRHW) {
+      if (m.E > (int64_t)g_vol_[1] * kWarps) {
+        if constexpr (kVolRW) {
+          using R = VolR<D, K, false, true>;
+          launch(k_volume_r<D, K, false, false, true>, clamp_grid(g_volw_, (m.E + R::ELW - 1) / R::ELW, 1),
+                 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL), static_cast<const float*>(wL),
+                 static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
+        } else {
+          using R = VolRH<D, K, true>;
+          launch(k_volume_rh<D, K, true>, clamp_grid(g_volw_, (m.E + R::ELW - 1) / R::ELW, 1), 32 * R::WARPS, R::SMEM,
+                 st, m, t, static_cast<const float*>(uL), static_cast<const float*>(wL),
+                 static_cast<const float*>(gam), static_cast<float*>(out), c);
+        }
+        return 1;
+      }
+      launch(k_volume<D, K, T, true, kVolumeTab, false>, g, 32 * kWarps, volume_smem(true), st,
           m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(gam),
           static_cast<T*>(out), c, nullptr);
-    else
-      launch(k_volume<D, K, T, false, kVolumeTab, false>, g, 32 * kWarps, volume_smem(false), st, 
-          m, t, static_cast<const T*>(uL), static_cast<const T*>(uL), static_cast<const T*>(gam),
-          static_cast<T*>(out), c, nullptr);
+    } else {
+      if (wsep)
+        launch(k_volume<D, K, T, true, kVolumeTab, false>, g, 32 * kWarps, volume_smem(true), st,
+            m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(gam),
+            static_cast<T*>(out), c, nullptr);
+      else
+        launch(k_volume<D, K, T, false, kVolumeTab, false>, g, 32 * kWarps, volume_smem(false), st,
+            m, t, static_cast<const T*>(uL), static_cast<const T*>(uL), static_cast<const T*>(gam),
+            static_cast<T*>(out), c, nullptr);
+    }
     return 1;
   }
 
@@ -484,8 +523,8 @@ class OpsImpl final : public Ops {
       if (vvar_ == kVolRegFused) {
         using R = VolR<D, K>;
         const int g = clamp_grid(g_volrf_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_r<D, K, true, false>, g, 32 * R::WARPS, R::SMEM_FUSE, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(gam), static_cast<float*>(outV), c, static_cast<float*>(lf));
+        launch(k_volume_r<D, K, true, false, false>, g, 32 * R::WARPS, R::SMEM_FUSE, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(outV), c, static_cast<float*>(lf));
         return 1;
       }
     }

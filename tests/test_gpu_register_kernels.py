@@ -31,6 +31,20 @@ def _setup(dim, n, k, walls):
     topo = mesh.MeshTopo(m.coords, m.elems, rep)
     return g, topo, fe.ref_element(dim, k)
 
+# past one element per resident warp, where the separate-wind volume term changes kernels
+LARGER = [(2, 41, 2), (3, 8, 2), (3, 9, 3), (3, 8, 4), (3, 6, 5)]
+
+
+@pytest.mark.parametrize("dim,n,k", LARGER)
+def test_separate_wind_volume_kernels(dim, n, k):
+    g, topo, ref = _setup(dim, n, k, False)
+    sp = hdiv.HDiv(topo, ref)
+    rng = np.random.default_rng(7500 + 10 * dim + k)
+    wV, u = (rng.standard_normal(s).astype(np.float32).astype(np.float64) for s in (sp.n_hdiv, (topo.n_elems, dim, ref.nb)))
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x).reshape(-1), dtype=torch.float32, device=g.device)  # noqa: E731
+    y = g.apply_convection(dev(wV), dev(u))
+    assert _rel(y, C.apply(topo, ref, sp.to_l2(wV), u, k - 1)) < 1e-6
+
 
 @pytest.mark.parametrize("walls", [False, True])
 @pytest.mark.parametrize("dim,n,k", ORDERS)
