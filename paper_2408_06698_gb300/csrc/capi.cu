@@ -1278,7 +1278,9 @@ hopu_status hopu_vjp_apply(hopu_ctx* c, const void* w_hdiv, const void* u_l2, co
   hopu_status r = ensure_gamW(c);
   if (r != HOPU_OK) return r;
   enqueue_v2l(c, w_hdiv, c->d_wL);
-  enqueue_apply_vjp(c, u_l2, c->d_wL, ybar_l2, ubar_l2 ? ubar_l2 : c->d_uL, c->d_yL);
+  // FP32 runs one kernel per cotangent and skips the one not asked for
+  enqueue_apply_vjp(c, u_l2, c->d_wL, ybar_l2, ubar_l2 ? ubar_l2 : (c->fp64 ? c->d_uL : nullptr),
+                    wbar_hdiv || c->fp64 ? c->d_yL : nullptr);
   if (wbar_hdiv) {
     Combine plain;
     enqueue_l2v(c, c->d_yL, true, plain, wbar_hdiv);

@@ -66,39 +66,122 @@ struct FacR {
   static constexpr int MINB = REGS <= 120 ? 3 : 2;
 };
 
+// Both sides' records of a group's facets into the warp's buffer: record r < FPW is side A of
+// facet r, record FPW + r its side B (pa, pb: this lane's facet's elements * 4 + f).  A record is
+// copied by CH lanes, RPI records per step, as the 16-byte chunks that hold it.
+template <int D, int K>
+__device__ __forceinline__ void facet_request(const float* src, float* sRec, int pa, int pb, int lane) {
+  using C = FacR<D, K>;
+  constexpr int NL = C::NL, FPW = C::FPW, CH = C::CH, RST = C::RST;
+  constexpr int RPI = CH <= 16 ? (CH <= 8 ? 4 : 2) : 1, LPR = 32 / RPI;
+  const int cr = lane / LPR, cc0 = lane - cr * LPR;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const int ids = (side ? pb : pa) >> 2;
+#pragma unroll 5
+    for (int r0 = 0; r0 < FPW; r0 += RPI) {
+      const int r = r0 + cr;
+      const int64_t start = (int64_t)__shfl_sync(kFull, ids, r * D & 31) * NL;
+      const int shift = NL % 4 ? int(start & 3) : 0;
+      float* dst = sRec + (side * FPW + r) * RST;
+#pragma unroll
+      for (int c = cc0; c < ((CH + LPR - 1) / LPR) * LPR; c += LPR) {
+        const int left = shift + NL - 4 * c;  // floats up to the record's end
+        if (r < FPW && left > 0) {
+          if (NL % 4) cp_async_part(dst + 4 * c, src + (start - shift) + 4 * c, left < 4 ? 4 * left : 16);
+          else cp_async<16>(dst + 4 * c, src + start + 4 * c);
+        }
+      }
+    }
+  }
+  cp_commit();
+}
+
+// Component a of facet fl's record of one side, as pairs of neighbouring basis indices.
+template <int D, int K>
+__device__ __forceinline__ void facet_take(const float* sRec, int side, int fl, int a, int64_t e,
+                                           f2 (&c)[FacR<D, K>::NBP]) {
+  using C = FacR<D, K>;
+  constexpr int NB = C::NB, NL = C::NL;
+  const float* p = sRec + (side * C::FPW + fl) * C::RST + a * NB;
+  if constexpr (NL % 4 == 0 && NB % 4 == 0) {
+#pragma unroll
+    for (int j = 0; j < C::NBP; j += 2) lds_f2(p + 2 * j, c[j], c[j + 1]);
+  } else {
+    if (NL % 4) p += (e * NL) & 3;
+#pragma unroll
+    for (int j = 0; j < C::NBP; ++j) c[j] = f2_pack(p[2 * j], 2 * j + 1 < NB ? p[2 * j + 1] : 0.0f);
+  }
+}
+
+// Plain part of mode mm's trace (row: TrM[f][mm]) from the basis indices that have one: those of
+// the mode's degree on, and, unless all are wanted, past the compensated ones (i <= D) for the
+// modes of degree <= 1.
+template <int D, int K>
+__device__ __forceinline__ float facet_plain_trace(int mm, const float* row, const f2 (&c)[FacR<D, K>::NBP], bool all) {
+  constexpr int NB = FacR<D, K>::NB, NBP = FacR<D, K>::NBP;
+  const int n = mode_degree(D - 1, mm);
+  const int i0 = (n <= 1 && !all) ? D + 1 : cnbasis(D, n - 1);
+  f2 s = f2_zero();
+  float odd = 0.0f;
+#pragma unroll
+  for (int i = 0; i < NB; i += 4)
+    if (i + 4 > i0) {
+      f2 t[2];
+      lds_f2(row + i, t[0], t[1]);
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const int j = i + 2 * w;
+        if (j >= NB || j + 2 <= i0) continue;
+        const f2 cj = c[j / 2 < NBP ? j / 2 : 0];
+        if (j < i0) odd = f2_y(t[w]) * f2_y(cj);
+        else s = f2_fma(t[w], cj, s);
+      }
+    }
+  return (i0 & 1) ? f2_sum(s) + odd : f2_sum(s);
+}
+
+// Tables of a facet kernel: trace matrices, the point factors A and B (each value twice), w_q / 2.
+template <int D, int K>
+__device__ __forceinline__ void facet_stage_tables(const DevTabs& tb, float* sm) {
+  using C = FacR<D, K>;
+  constexpr int NB = C::NB, NF = C::NF, NB4 = C::NB4, MF = C::MF, AST = C::AST, BST = C::BST;
+  const float* TrMg = static_cast<const float*>(tb.TrM);
+  const float* FAg = static_cast<const float*>(tb.FacA);  // [MF][K+1]
+  const float* FBg = static_cast<const float*>(tb.FacB);  // [MF][NF]
+  const float* Wfg = static_cast<const float*>(tb.Wf);
+  for (int t = threadIdx.x; t < (D + 1) * NF * NB4; t += blockDim.x) {
+    const int row = t / NB4, i = t - row * NB4;
+    sm[C::O_TRM + t] = i < NB ? TrMg[row * NB + i] : 0.0f;
+  }
+  for (int t = threadIdx.x; t < (D + 1) * (D + 1) * 4; t += blockDim.x) {
+    const int mm = t & 3, i = (t >> 2) % (D + 1), f = (t >> 2) / (D + 1);
+    sm[C::O_LOW + t] = mm < NF ? TrMg[(f * NF + mm) * NB + i] : 0.0f;
+  }
+  for (int t = threadIdx.x; t < MF * AST; t += blockDim.x) {
+    const int i = t / AST, p = (t - i * AST) >> 1;
+    sm[C::O_A + t] = p <= K ? FAg[i * (K + 1) + p] : 0.0f;
+  }
+  if constexpr (D == 3) {
+    for (int t = threadIdx.x; t < MF * BST; t += blockDim.x) {
+      const int j = t / BST, mm = (t - j * BST) >> 1;
+      sm[C::O_B + t] = mm < NF ? FBg[j * NF + mm] : 0.0f;
+    }
+  }
+  for (int t = threadIdx.x; t < C::NQF; t += blockDim.x)
+    sm[C::O_WF + t] = 0.5f * Wfg[D == 3 ? (t % MF) * MF + t / MF : t];  // rule order: q = i MF + j
+}
+
 template <int D, int K, bool WSEP>
 __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
     k_facet_r(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ wL, int lconst,
               const int8_t* __restrict__ facet_l, float* __restrict__ gam, double* __restrict__ diss) {
   using C = FacR<D, K>;
-  constexpr int NB = C::NB, NF = C::NF, NL = C::NL, NQF = C::NQF, NB4 = C::NB4, FPW = C::FPW;
-  constexpr int NBP = C::NBP, CH = C::CH, RST = C::RST, MF = C::MF, AST = C::AST, BST = C::BST;
+  constexpr int NF = C::NF, NB4 = C::NB4, FPW = C::FPW, NBP = C::NBP, RST = C::RST;
+  constexpr int MF = C::MF, AST = C::AST, BST = C::BST;
   extern __shared__ __align__(16) float sm[];
   pdl_trigger();
-  {
-    const float* TrMg = static_cast<const float*>(tb.TrM);
-    const float* FAg = static_cast<const float*>(tb.FacA);    // [MF][K+1]
-    const float* FBg = static_cast<const float*>(tb.FacB);    // [MF][NF]
-    const float* Wfg = static_cast<const float*>(tb.Wf);
-    for (int t = threadIdx.x; t < (D + 1) * NF * NB4; t += blockDim.x) {
-      const int row = t / NB4, i = t - row * NB4;
-      sm[C::O_TRM + t] = i < NB ? TrMg[row * NB + i] : 0.0f;
-    }
-    for (int t = threadIdx.x; t < (D + 1) * (D + 1) * 4; t += blockDim.x) {
-      const int mm = t & 3, i = (t >> 2) % (D + 1), f = (t >> 2) / (D + 1);
-      sm[C::O_LOW + t] = mm < NF ? TrMg[(f * NF + mm) * NB + i] : 0.0f;
-    }
-    for (int t = threadIdx.x; t < MF * AST; t += blockDim.x) {
-      const int i = t / AST, p = (t - i * AST) >> 1;
-      sm[C::O_A + t] = p <= K ? FAg[i * (K + 1) + p] : 0.0f;
-    }
-    for (int t = threadIdx.x; t < MF * BST; t += blockDim.x) {
-      const int j = t / BST, mm = (t - j * BST) >> 1;
-      sm[C::O_B + t] = mm < NF ? FBg[j * NF + mm] : 0.0f;
-    }
-    for (int t = threadIdx.x; t < NQF; t += blockDim.x)
-      sm[C::O_WF + t] = 0.5f * Wfg[D == 3 ? (t % MF) * MF + t / MF : t];  // rule order: q = i MF + j
-  }
+  facet_stage_tables<D, K>(tb, sm);
   const float* sTrM = sm + C::O_TRM;
   const float* sLow = sm + C::O_LOW;
   const float* sA = sm + C::O_A;
@@ -118,67 +201,10 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
     return s;
   };
   const int64_t ngroups = (m.NF + FPW - 1) / FPW, gstep = (int64_t)gridDim.x * C::WARPS;
-  // both sides' records of a group's facets into the warp's buffer: record r < FPW is side A
-  // of facet r, record FPW + r its side B (pa, pb: this lane's facet's elements * 4 + f); a
-  // record is copied by CH lanes, RPI records per step
-  constexpr int RPI = CH <= 16 ? (CH <= 8 ? 4 : 2) : 1, LPR = 32 / RPI;
-  const int cr = lane / LPR, cc0 = lane - cr * LPR;
-  auto request = [&](const float* src, int pa, int pb) {
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const int ids = (side ? pb : pa) >> 2;
-#pragma unroll 5
-      for (int r0 = 0; r0 < FPW; r0 += RPI) {
-        const int r = r0 + cr;
-        const int64_t start = (int64_t)__shfl_sync(kFull, ids, r * D & 31) * NL;
-        const int shift = NL % 4 ? int(start & 3) : 0;
-        float* dst = sRec + (side * FPW + r) * RST;
-#pragma unroll
-        for (int c = cc0; c < ((CH + LPR - 1) / LPR) * LPR; c += LPR) {
-          const int left = shift + NL - 4 * c;  // floats up to the record's end
-          if (r < FPW && left > 0) {
-            if (NL % 4) cp_async_part(dst + 4 * c, src + (start - shift) + 4 * c, left < 4 ? 4 * left : 16);
-            else cp_async<16>(dst + 4 * c, src + start + 4 * c);
-          }
-        }
-      }
-    }
-    cp_commit();
-  };
-  // this lane's component of one side's record, as pairs of neighbouring basis indices
-  auto take = [&](int side, int64_t e, f2 (&c)[NBP]) {
-    const float* p = sRec + (side * FPW + fl) * RST + a * NB;
-    if constexpr (NL % 4 == 0 && NB % 4 == 0) {
-#pragma unroll
-      for (int j = 0; j < NBP; j += 2) lds_f2(p + 2 * j, c[j], c[j + 1]);
-    } else {
-      if (NL % 4) p += (e * NL) & 3;
-#pragma unroll
-      for (int j = 0; j < NBP; ++j) c[j] = f2_pack(p[2 * j], 2 * j + 1 < NB ? p[2 * j + 1] : 0.0f);
-    }
-  };
-  // plain part of mode mm's trace from the basis indices that have one: those of the mode's
-  // degree on, and past the compensated ones (i <= D) for the modes of degree <= 1
-  auto plain = [&](int mm, const float* row, const f2 (&c)[NBP], bool all) -> float {
-    const int n = mode_degree(D - 1, mm);
-    const int i0 = (n <= 1 && !all) ? D + 1 : cnbasis(D, n - 1);
-    f2 s = f2_zero();
-    float odd = 0.0f;
-#pragma unroll
-    for (int i = 0; i < NB; i += 4)
-      if (i + 4 > i0) {
-        f2 t[2];
-        lds_f2(row + i, t[0], t[1]);
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-          const int j = i + 2 * w;
-          if (j >= NB || j + 2 <= i0) continue;
-          const f2 cj = c[j / 2 < NBP ? j / 2 : 0];
-          if (j < i0) odd = f2_y(t[w]) * f2_y(cj);
-          else s = f2_fma(t[w], cj, s);
-        }
-      }
-    return (i0 & 1) ? f2_sum(s) + odd : f2_sum(s);
+  auto request = [&](const float* src, int pa, int pb) { facet_request<D, K>(src, sRec, pa, pb, lane); };
+  auto take = [&](int side, int64_t e, f2 (&c)[NBP]) { facet_take<D, K>(sRec, side, fl, a, e, c); };
+  auto plain = [&](int mm, const float* row, const f2 (&c)[NBP], bool all) {
+    return facet_plain_trace<D, K>(mm, row, c, all);
   };
   int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x;
   int npa = 0, npb = 0;  // the next group's elements of this lane's facet

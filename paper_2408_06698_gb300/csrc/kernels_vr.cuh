@@ -29,10 +29,17 @@
 // each row, D staged per CTA, the shares summed by shuffles); interior rows are combined
 // into the V_h output, facet rows go to lf with the sign sigma.
 //
-// WSEP: a wind w of its own: lane a holds the modal coefficients of the reference component
+// Separate wind (kVolWind): lane a holds the modal coefficients of the reference component
 // W_a = sum_b M[a][b] w_b and those of div^ W = sum_a d^_a W_a (summed over the element's lanes
 // once), evaluates both at the points with the same basis row and takes the other W by
 // shuffles; one point per pass where the registers end (k = 4).
+//
+// VJP (kVolAdj*): the volume parts of the cotangents of u and w (kernels_adj.cuh) have the same
+// shape, the gradient taken of z = ybar / |det J| and the facet moments those of the adjoint
+// facet kernel; each cotangent is one run of the point loop, with w = u one for their sum.  A
+// single loop for both cotangents would hold two accumulator sets beside G, which ends the
+// registers at k = 3; the warp-per-element kernel that did so kept its 2 x 64 sums in local
+// memory (16^3 x 6, k = 3: 1272 us against 61 us for the two launches; k = 4: 4045 against 178).
 //
 // Bound: the FMA units' register reads (three distinct 64-bit operands per paired FMA: a copy
 // of the inner loop alone ran at 210 cycles per point and warp at k = 4, against 139 of FMA
@@ -47,7 +54,16 @@
 
 namespace hopu {
 
-template <int D, int K, bool GTAB = false, bool WSEP = false>
+// What the point loop of the register volume kernels evaluates and tests.
+enum VolMode {
+  kVolSame = 0,     // y: w = u
+  kVolWind = 1,     // y: separate wind
+  kVolAdjU = 2,     // VJP, cotangent of u: f = -W . grad^ z
+  kVolAdjW = 3,     // VJP, cotangent of w: f = -sum_c M[c][a] sum_b u_b d^_c z_b
+  kVolAdjSame = 4   // VJP with w = u: the sum of both
+};
+
+template <int D, int K, bool GTAB = false, int MODE = kVolSame>
 struct VolR {
   using S = Shape<D, K>;
   static constexpr int NB = S::nb, NB1 = cnbasis(D, K - 1), NF = S::nf, NL = S::nloc, NQ = S::nq, GT = S::gt;
@@ -64,13 +80,15 @@ struct VolR {
   static constexpr int O_W = O_TRM + (D + 1) * NF * NB4;
   static constexpr int PER_WARP = r4i(ELW * NL);     // the warp's element records: in, and out
   static constexpr int GW = r4i(ELW * NG);           // the warp's facet moments
-  static constexpr int O_G = O_W + WARPS * (WSEP ? 3 : 2) * PER_WARP;
-  static constexpr size_t SMEM = size_t(O_G + WARPS * GW) * 4;
+  static constexpr int NBUF = MODE == kVolSame ? 2 : 3;  // records: in (one or two fields), out
+  static constexpr int NGAM = MODE == kVolAdjSame ? 2 : 1;
+  static constexpr int O_G = O_W + WARPS * NBUF * PER_WARP;
+  static constexpr size_t SMEM = size_t(O_G + WARPS * NGAM * GW) * 4;
   static constexpr int NLR = row_stride<float>(NL);  // rows of the row-major D in global memory
   static constexpr int NDP = D * NB4;                // fused back-projection: D [NL][D blocks of NB4]
   static constexpr int O_D = O_G + WARPS * GW;
   static constexpr size_t SMEM_FUSE = size_t(O_D + NL * NDP) * 4;
-  static constexpr int REGS = (WSEP ? 3 * NB + NB1 : 2 * NB) + (GTAB ? 0 : D * NB1);  // c, r, G of a lane (and w, div w)
+  static constexpr int REGS = (MODE == kVolWind ? 3 * NB + NB1 : 2 * NB) + (GTAB ? 0 : D * NB1);  // c, r, G of a lane (and w, div w)
   static constexpr int XP = REGS <= 140 ? 2 : 1;  // quadrature points per pass
   static constexpr int MINB = GTAB ? 2 : (REGS <= 90 ? 3 : 2);  // resident CTAs asked of the register allocator
   static constexpr bool OK = REGS <= 190 && SMEM <= 200 * 1024;
@@ -90,11 +108,16 @@ __device__ __forceinline__ void warp_copy_records(float* dst, const float* src, 
   }
 }
 
-template <int D, int K, bool FUSE, bool GTAB, bool WSEP>
-__global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K, GTAB, WSEP>::MINB)
-    k_volume_r(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ wL,
-               const float* __restrict__ gam, float* out, Combine cmb, float* __restrict__ lf) {
-  using C = VolR<D, K, GTAB, WSEP>;
+// in1: the field evaluated at the points (u; the wind for kVolAdjU); in2: the wind (kVolWind) or
+// the cotangent ybar (VJP); gam2: the wind's moments (kVolAdjSame).
+template <int D, int K, bool FUSE, bool GTAB, int MODE>
+__global__ void __launch_bounds__(32 * VolR<D, K, GTAB, MODE>::WARPS, VolR<D, K, GTAB, MODE>::MINB)
+    k_volume_r(DevMesh m, DevTabs tb, const float* __restrict__ in1, const float* __restrict__ in2,
+               const float* __restrict__ gam, const float* __restrict__ gam2, float* out, Combine cmb,
+               float* __restrict__ lf) {
+  using C = VolR<D, K, GTAB, MODE>;
+  constexpr bool WIND = MODE == kVolWind, ADJ = MODE >= kVolAdjU;
+  constexpr bool ROW = WIND || MODE == kVolAdjU;   // the wind enters through its reference components
   using S = Shape<D, K>;
   constexpr int NB = C::NB, NB1 = C::NB1, NF = C::NF, NL = C::NL, NQ = C::NQ, GT = C::GT;
   constexpr int NBQ = C::NBQ, NB4 = C::NB4, NG = C::NG, ELW = C::ELW, NP = C::NP, NP1 = C::NP1;
@@ -141,16 +164,16 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
   // the other lanes of the element (idle lanes talk to themselves)
   const int p1 = lane_on ? el * D + a1 : lane;
   const int p2 = lane_on ? el * D + a2 : lane;
-  float* sIn = sm + C::O_W + warp * (WSEP ? 3 : 2) * C::PER_WARP;
+  float* sIn = sm + C::O_W + warp * C::NBUF * C::PER_WARP;
   float* sY = sIn + C::PER_WARP;
-  float* sWn = sY + (WSEP ? C::PER_WARP : 0);  // the wind's records (WSEP)
-  float* sG = sm + C::O_G + warp * C::GW;
+  float* sIn2 = sY + (MODE == kVolSame ? 0 : C::PER_WARP);
+  float* sG = sm + C::O_G + warp * C::NGAM * C::GW;
   const int64_t ngroups = (m.E + ELW - 1) / ELW, gstep = (int64_t)gridDim.x * C::WARPS;
   auto count = [&](int64_t g) { return (m.E - g * ELW < ELW) ? (int)(m.E - g * ELW) : ELW; };
   int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x;
   auto request = [&](int64_t g) {
-    warp_copy_records<NL, ELW>(sIn, uL, g * ELW, count(g), lane);
-    if (WSEP) warp_copy_records<NL, ELW>(sWn, wL, g * ELW, count(g), lane);
+    warp_copy_records<NL, ELW>(sIn, in1, g * ELW, count(g), lane);
+    if (MODE != kVolSame) warp_copy_records<NL, ELW>(sIn2, in2, g * ELW, count(g), lane);
   };
   if (grp < ngroups) request(grp);
   cp_commit();
@@ -160,40 +183,52 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
     const bool act = lane_on && el < ne;
     const int64_t e = act ? e0 + el : e0;  // inactive lanes read the group's first element
     const double* gp = m.geoT + e * GT;
-    // M = |det J| J^-1: its columns a, a + 1, a + 2 (w = u), or its row a in M0 (separate wind)
-    float M0[D], M1[WSEP ? 1 : D], M2[WSEP ? 1 : D];
+    // M = |det J| J^-1: its columns a, a + 1, a + 2 (w = u), column a (kVolAdjW) or row a in M0
+    constexpr bool COLS = MODE == kVolSame || MODE == kVolAdjSame;
+    float M0[D], M1[COLS ? D : 1], M2[COLS ? D : 1];
 #pragma unroll
     for (int cc = 0; cc < D; ++cc) {
-      M0[cc] = float(__ldg(gp + 2 * D * D + (WSEP ? a * D + cc : cc * D + a)));
-      if constexpr (!WSEP) {
+      M0[cc] = float(__ldg(gp + 2 * D * D + (ROW ? a * D + cc : cc * D + a)));
+      if constexpr (COLS) {
         M1[cc] = float(__ldg(gp + 2 * D * D + cc * D + a1));
         M2[cc] = D == 3 ? float(__ldg(gp + 2 * D * D + cc * D + a2)) : 0.0f;
       }
     }
     const float invabs = float(__ldg(gp + 3 * D * D));
-    f2 c[NP], cw[WSEP ? NP : 1];
+    // c: the coefficients whose gradient is taken (u; z = ybar / |det J| in the VJP);
+    // ev: those evaluated at the points (c itself when w = u; the modal W_a = sum_b M[a][b] w_b,
+    // the wind's reference component a; u in the wind's cotangent)
+    f2 c[NP], ev[MODE == kVolSame ? 1 : NP];
     cp_wait<0>();
     __syncwarp();
     {
-      const int o = ((act ? el : 0) * D + a) * NB;
+      const int oe = (act ? el : 0) * NL, o = oe + a * NB;
+      const float* sC = ADJ ? sIn2 : sIn;
+      const float sc = ADJ ? invabs : 1.0f;
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
-        c[j] = f2_pack(sIn[o + 2 * j], 2 * j + 1 < NB ? sIn[o + 2 * j + 1] : 0.0f);
-        if constexpr (WSEP) {  // modal W_a = sum_b M[a][b] w_b, the wind's reference component a
+        const bool pair = 2 * j + 1 < NB;
+        c[j] = f2_pack(sC[o + 2 * j], pair ? sC[o + 2 * j + 1] : 0.0f);
+        if constexpr (ADJ) c[j] = f2_mul(c[j], f2_dup(sc));
+        if constexpr (ROW) {
+          const float* sWn = WIND ? sIn2 : sIn;
           float v[2] = {0.0f, 0.0f};
 #pragma unroll
           for (int w = 0; w < 2; ++w)
             if (2 * j + w < NB) {
 #pragma unroll
-              for (int b = 0; b < D; ++b) v[w] = fmaf(M0[b], sWn[((act ? el : 0) * D + b) * NB + 2 * j + w], v[w]);
+              for (int b = 0; b < D; ++b) v[w] = fmaf(M0[b], sWn[oe + b * NB + 2 * j + w], v[w]);
             }
-          cw[j] = f2_pack(v[0], v[1]);
+          ev[j] = f2_pack(v[0], v[1]);
+        } else if constexpr (ADJ) {
+          ev[j] = f2_pack(sIn[o + 2 * j], pair ? sIn[o + 2 * j + 1] : 0.0f);
         }
       }
     }
     __syncwarp();
     // this group's facet moments and the next group's coefficients arrive during the points
     warp_copy_records<NG, ELW>(sG, gam, e0, ne, lane);
+    if (MODE == kVolAdjSame) warp_copy_records<NG, ELW>(sG + C::GW, gam2, e0, ne, lane);
     if (grp + gstep < ngroups) request(grp + gstep);
     cp_commit();
     // entry `row` of the modal reference derivative Dm_cc of the coefficients x
@@ -213,11 +248,11 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
       return f2_sum(s);
     };
     // separate wind: modal coefficients of div^ W = sum_a d^_a W_a, a term from each lane
-    f2 dw[WSEP ? NP1 : 1];
-    if constexpr (WSEP) {
+    f2 dw[WIND ? NP1 : 1];
+    if constexpr (WIND) {
       float pd[NB1];
 #pragma unroll
-      for (int j = 0; j < NB1; ++j) pd[j] = derivative(cw, a, j);
+      for (int j = 0; j < NB1; ++j) pd[j] = derivative(ev, a, j);
       __syncwarp();  // keeps the products of the two derivatives apart (registers)
 #pragma unroll
       for (int j = 0; j < NB1; ++j) {
@@ -245,10 +280,12 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
     // two points per pass where the registers allow it: the loads and shuffles of one overlap
     // the arithmetic of the other (an odd last point is paired with itself at weight 0)
     constexpr int XP = C::XP;
-    // Separate wind, many points: the test sums run in blocks of points whose partial sums meet
-    // in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
-    // more than the warp-per-element kernel, whose points are summed pairwise.
-    constexpr int QB = (WSEP && NQ > 64) ? (NQ / 8 + 1) * 2 : NQ;
+    // Separate wind and VJP, many points: the test sums run in blocks of points whose partial sums
+    // meet in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
+    // more than a warp per element, whose points are summed pairwise; one over 46 points rounded
+    // the wind's cotangent 20 % more (at k = 3 the blocks cost 5 us of 61).
+    constexpr int QLIM = MODE == kVolWind ? 64 : (MODE == kVolAdjSame ? 100 : 16);
+    constexpr int QB = (MODE != kVolSame && NQ > QLIM) ? (NQ / 8 + 1) * 2 : NQ;
     float* yp = sY + ((act ? el : 0) * D + a) * NB;  // this lane's output entries
 #pragma unroll 1
     for (int q0 = 0; q0 < NQ; q0 += QB) {
@@ -275,9 +312,11 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
 #pragma unroll
               for (int w = 0; w < 2; ++w) {
                 const int j = i / 2 + w;
-                if (j < NP) us[x] = f2_fma(t[w], c[j < NP ? j : 0], us[x]);
-                if constexpr (WSEP) {
-                  if (j < NP) ws[x] = f2_fma(t[w], cw[j < NP ? j : 0], ws[x]);
+                if (!ADJ && j < NP) us[x] = f2_fma(t[w], c[j < NP ? j : 0], us[x]);
+                if constexpr (MODE != kVolSame) {
+                  if (j < NP) ws[x] = f2_fma(t[w], ev[j < NP ? j : 0], ws[x]);
+                }
+                if constexpr (WIND) {
                   if (j < NP1) ds[x] = f2_fma(t[w], dw[j < NP1 ? j : 0], ds[x]);
                 }
                 if constexpr (!GTAB) {
@@ -305,7 +344,7 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
 #pragma unroll
           for (int x = 0; x < XP; ++x) {
             u[x] = f2_sum(us[x]);
-            wa[x] = WSEP ? f2_sum(ws[x]) : u[x];
+            wa[x] = MODE == kVolSame ? u[x] : f2_sum(ws[x]);
             dvs[x] = f2_sum(ds[x]);
 #pragma unroll
             for (int cc = 0; cc < D; ++cc) gd[x][cc] = f2_sum(gs[x][cc]);
@@ -314,28 +353,41 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
         f2 ff[XP];
 #pragma unroll
         for (int x = 0; x < XP; ++x) {
-          float f;
-          if constexpr (WSEP) {
-            f = dvs[x] * u[x];
+          float f = 0.0f;
+          if constexpr (ROW) {  // (div^ W) u_a + W . grad^ u_a, or - W . grad^ z_a
+            if (WIND) f = dvs[x] * u[x];
 #pragma unroll
             for (int cc = 0; cc < D; ++cc) f = fmaf(__shfl_sync(kFull, wa[x], el * D + cc), gd[x][cc], f);
-          } else {
-            // W = M u with the other components' u; div^ W = sum_b sum_c M[c][b] d^_c u_b
-            const float u1 = __shfl_sync(kFull, u[x], p1);
-            const float u2 = D == 3 ? __shfl_sync(kFull, u[x], p2) : 0.0f;
+          }
+          if constexpr (MODE == kVolSame) {
+            // div^ W = sum_b sum_c M[c][b] d^_c u_b
             float pd = 0.0f;
 #pragma unroll
             for (int cc = 0; cc < D; ++cc) pd = fmaf(M0[cc], gd[x][cc], pd);
             float dv = pd + __shfl_sync(kFull, pd, p1);
             if (D == 3) dv += __shfl_sync(kFull, pd, p2);
             f = dv * u[x];
+          }
+          if constexpr (COLS) {  // W = M u with the other components' u
+            const float u1 = __shfl_sync(kFull, wa[x], p1);
+            const float u2 = D == 3 ? __shfl_sync(kFull, wa[x], p2) : 0.0f;
 #pragma unroll
             for (int cc = 0; cc < D; ++cc) {
-              float W = fmaf(M1[cc], u1, M0[cc] * u[x]);
+              float W = fmaf(M1[cc], u1, M0[cc] * wa[x]);
               if (D == 3) W = fmaf(M2[cc], u2, W);
               f = fmaf(W, gd[x][cc], f);
             }
           }
+          if constexpr (MODE == kVolAdjW || MODE == kVolAdjSame) {  // sum_c M[c][a] sum_b u_b d^_c z_b
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) {
+              const float v = wa[x] * gd[x][cc];
+              float ug = v + __shfl_sync(kFull, v, p1);
+              if (D == 3) ug += __shfl_sync(kFull, v, p2);
+              f = fmaf(M0[cc], ug, f);
+            }
+          }
+          if (ADJ) f = -f;
           ff[x] = f2_dup(f * (x == 0 || two ? sWq[qs[x]] : 0.0f));
         }
 #pragma unroll
@@ -372,7 +424,8 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
       for (int f = 0; f <= D; ++f) {
 #pragma unroll
         for (int mm = 0; mm < NF; ++mm) {
-          const f2 gv = f2_dup(gl[(f * NF + mm) * D]);
+          const f2 gv = f2_dup(MODE == kVolAdjSame ? gl[(f * NF + mm) * D] + gl[C::GW + (f * NF + mm) * D]
+                                                 : gl[(f * NF + mm) * D]);
           const int i0 = cnbasis(D, mode_degree(D - 1, mm) - 1);  // lower degrees have no such trace
           const float* trow = sTrM + (f * NF + mm) * NB4;
 #pragma unroll
@@ -399,8 +452,8 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, WSEP>::WARPS, VolR<D, K,
     if (act) {
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
-        yp[2 * j] = f2_x(r[j]) * invabs;
-        if (2 * j + 1 < NB) yp[2 * j + 1] = f2_y(r[j]) * invabs;
+        yp[2 * j] = f2_x(r[j]) * (ADJ ? 1.0f : invabs);
+        if (2 * j + 1 < NB) yp[2 * j + 1] = f2_y(r[j]) * (ADJ ? 1.0f : invabs);
       }
     }
     __syncwarp();

@@ -12,7 +12,7 @@
 // accumulate their own r_i.  The tables are staged with their basis columns permuted so that
 // each half reads one contiguous block of a row (half h at column offset h HP).  Half the
 // registers per lane of k_volume_r: a register kernel at k = 5, where a whole basis does not
-// fit in one lane.  WSEP: a wind of its own, as in k_volume_r.
+// fit in one lane.  Separate wind and VJP as in k_volume_r.
 //
 // Bound: FMA register reads and the shuffles.  Measured (CUDA events, per launch): 18^3 x 6,
 // k = 5, w = u 437 -> 351 us (scalar FMAs, dense Dm and TrM products before); 13^3 x 6, k = 5,
@@ -24,7 +24,7 @@
 
 namespace hopu {
 
-template <int D, int K, bool WSEP = false>
+template <int D, int K, int MODE = kVolSame>
 struct VolRH {
   using S = Shape<D, K>;
   static constexpr int NB = S::nb, NB1 = cnbasis(D, K - 1), NF = S::nf, NL = S::nloc, NQ = S::nq, GT = S::gt;
@@ -43,21 +43,26 @@ struct VolRH {
   static constexpr int O_W = O_TRM + (D + 1) * NF * RW;
   static constexpr int PER_WARP = r4i(ELW * NL);  // the warp's element records: in (u, w), and out
   static constexpr int GW = r4i(ELW * NG);        // the warp's facet moments
-  static constexpr int NBUF = WSEP ? 3 : 2;
-  // tables above 64 KB: one CTA of 8 warps per SM; else CTAs of 4 warps, as many as fit
-  static constexpr int WARPS = O_W * 4 > 64 * 1024 ? 8 : 4;
+  static constexpr int NBUF = MODE == kVolSame ? 2 : 3;
+  static constexpr int NGAM = MODE == kVolAdjSame ? 2 : 1;
+  // tables above 64 KB: one CTA of 8 warps (6 with two sets of moments) per SM; else CTAs of 4
+  // warps, as many as fit
+  static constexpr int WARPS = O_W * 4 > 64 * 1024 ? (NGAM == 2 ? 6 : 8) : 4;
   static constexpr int O_G = O_W + WARPS * NBUF * PER_WARP;
-  static constexpr size_t SMEM = size_t(O_G + WARPS * GW) * 4;
-  static constexpr int REGS = (WSEP ? 3 * NH + NH1 : 2 * NH) + D * NH1;  // a lane's vectors
-  static constexpr int MINB = WARPS == 8 ? 1 : (REGS <= 60 ? 4 : 3);
+  static constexpr size_t SMEM = size_t(O_G + WARPS * NGAM * GW) * 4;
+  static constexpr int REGS = (MODE == kVolWind ? 3 * NH + NH1 : 2 * NH) + D * NH1;  // a lane's vectors
+  static constexpr int MINB = WARPS > 4 ? 1 : (REGS <= 60 ? 4 : 3);
   static constexpr bool OK = REGS <= 160 && SMEM <= 220 * 1024 && NB >= 2;
 };
 
-template <int D, int K, bool WSEP>
-__global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSEP>::MINB)
-    k_volume_rh(DevMesh m, DevTabs tb, const float* __restrict__ uL, const float* __restrict__ wL,
-                const float* __restrict__ gam, float* out, Combine cmb) {
-  using C = VolRH<D, K, WSEP>;
+// Arguments as k_volume_r.
+template <int D, int K, int MODE>
+__global__ void __launch_bounds__(32 * VolRH<D, K, MODE>::WARPS, VolRH<D, K, MODE>::MINB)
+    k_volume_rh(DevMesh m, DevTabs tb, const float* __restrict__ in1, const float* __restrict__ in2,
+                const float* __restrict__ gam, const float* __restrict__ gam2, float* out, Combine cmb) {
+  using C = VolRH<D, K, MODE>;
+  constexpr bool WIND = MODE == kVolWind, ADJ = MODE >= kVolAdjU;
+  constexpr bool ROW = WIND || MODE == kVolAdjU;   // the wind enters through its reference components
   constexpr int NB = C::NB, NB1 = C::NB1, NF = C::NF, NL = C::NL, NQ = C::NQ, GT = C::GT;
   constexpr int NBQ = C::NBQ, HP = C::HP, RW = C::RW, NG = C::NG, ELW = C::ELW, LPE = C::LPE;
   constexpr int NH = C::NH, NH1 = C::NH1, NP = C::NP, NP1 = C::NP1;
@@ -102,13 +107,13 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
   const int p2 = lane_on ? el * LPE + a2 * 2 + h : lane;
   float* sIn = sm + C::O_W + warp * C::NBUF * C::PER_WARP;
   float* sY = sIn + C::PER_WARP;
-  float* sWn = sY + (WSEP ? C::PER_WARP : 0);
-  float* sG = sm + C::O_G + warp * C::GW;
+  float* sIn2 = sY + (MODE == kVolSame ? 0 : C::PER_WARP);
+  float* sG = sm + C::O_G + warp * C::NGAM * C::GW;
   const int64_t ngroups = (m.E + ELW - 1) / ELW, gstep = (int64_t)gridDim.x * C::WARPS;
   auto count = [&](int64_t g) { return (m.E - g * ELW < ELW) ? (int)(m.E - g * ELW) : ELW; };
   auto request = [&](int64_t g) {
-    warp_copy_records<NL, ELW>(sIn, uL, g * ELW, count(g), lane);
-    if (WSEP) warp_copy_records<NL, ELW>(sWn, wL, g * ELW, count(g), lane);
+    warp_copy_records<NL, ELW>(sIn, in1, g * ELW, count(g), lane);
+    if (MODE != kVolSame) warp_copy_records<NL, ELW>(sIn2, in2, g * ELW, count(g), lane);
   };
   auto halves = [&](float v) { return v + __shfl_sync(kFull, v, pt); };
   int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x;
@@ -120,42 +125,50 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
     const bool act = lane_on && el < ne;
     const int64_t e = act ? e0 + el : e0;  // inactive lanes read the group's first element
     const double* gp = m.geoT + e * GT;
-    // M = |det J| J^-1: its columns a, a + 1, a + 2 (w = u), or its row a in M0 (separate wind)
-    float M0[D], M1[WSEP ? 1 : D], M2[WSEP ? 1 : D];
+    // M = |det J| J^-1: its columns a, a + 1, a + 2 (w = u), column a (kVolAdjW) or row a in M0
+    constexpr bool COLS = MODE == kVolSame || MODE == kVolAdjSame;
+    float M0[D], M1[COLS ? D : 1], M2[COLS ? D : 1];
 #pragma unroll
     for (int cc = 0; cc < D; ++cc) {
-      M0[cc] = float(__ldg(gp + 2 * D * D + (WSEP ? a * D + cc : cc * D + a)));
-      if constexpr (!WSEP) {
+      M0[cc] = float(__ldg(gp + 2 * D * D + (ROW ? a * D + cc : cc * D + a)));
+      if constexpr (COLS) {
         M1[cc] = float(__ldg(gp + 2 * D * D + cc * D + a1));
         M2[cc] = D == 3 ? float(__ldg(gp + 2 * D * D + cc * D + a2)) : 0.0f;
       }
     }
     const float invabs = float(__ldg(gp + 3 * D * D));
-    // this half's coefficients, c_a[2 t + h] (zero beyond the half)
-    f2 c[NP], cw[WSEP ? NP : 1];
+    // this half's coefficients, entries 2 t + h (zero beyond the half): c those whose gradient is
+    // taken, ev those evaluated at the points (as in k_volume_r)
+    f2 c[NP], ev[MODE == kVolSame ? 1 : NP];
     cp_wait<0>();
     __syncwarp();
     {
-      const int o = ((act ? el : 0) * D + a) * NB + h;
+      const int oe = (act ? el : 0) * NL + h, o = oe + a * NB;
+      const float* sC = ADJ ? sIn2 : sIn;
+      const float sc = ADJ ? invabs : 1.0f;
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
-        const bool in0 = 2 * j < nh, in1 = 2 * j + 1 < nh;
-        c[j] = f2_pack(in0 ? sIn[o + 4 * j] : 0.0f, in1 ? sIn[o + 4 * j + 2] : 0.0f);
-        if constexpr (WSEP) {  // modal W_a = sum_b M[a][b] w_b, the wind's reference component a
+        const bool in0 = 2 * j < nh, in1_ = 2 * j + 1 < nh;
+        c[j] = f2_pack(in0 ? sC[o + 4 * j] : 0.0f, in1_ ? sC[o + 4 * j + 2] : 0.0f);
+        if constexpr (ADJ) c[j] = f2_mul(c[j], f2_dup(sc));
+        if constexpr (ROW) {
           float v[2] = {0.0f, 0.0f};
-          const float* wp = sWn + (act ? el : 0) * NL + h + 4 * j;
+          const float* wp = (WIND ? sIn2 : sIn) + oe + 4 * j;
 #pragma unroll
           for (int b = 0; b < D; ++b) {
             if (in0) v[0] = fmaf(M0[b], wp[b * NB], v[0]);
-            if (in1) v[1] = fmaf(M0[b], wp[b * NB + 2], v[1]);
+            if (in1_) v[1] = fmaf(M0[b], wp[b * NB + 2], v[1]);
           }
-          cw[j] = f2_pack(v[0], v[1]);
+          ev[j] = f2_pack(v[0], v[1]);
+        } else if constexpr (ADJ) {
+          ev[j] = f2_pack(in0 ? sIn[o + 4 * j] : 0.0f, in1_ ? sIn[o + 4 * j + 2] : 0.0f);
         }
       }
     }
     __syncwarp();
     // this group's facet moments and the next group's coefficients arrive during the points
     warp_copy_records<NG, ELW>(sG, gam, e0, ne, lane);
+    if (MODE == kVolAdjSame) warp_copy_records<NG, ELW>(sG + C::GW, gam2, e0, ne, lane);
     if (grp + gstep < ngroups) request(grp + gstep);
     cp_commit();
     // this half's entry j = 2 t + h of the modal reference derivative sum_i Dm[cc][j][i] x_i, xo
@@ -191,13 +204,13 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
         xo[j] = f2_pack(__shfl_sync(kFull, f2_x(x[j]), pt), __shfl_sync(kFull, f2_y(x[j]), pt));
     };
     // separate wind: this half's modal coefficients of div^ W = sum_a d^_a W_a, a term per lane
-    f2 dw[WSEP ? NP1 : 1];
-    if constexpr (WSEP) {
+    f2 dw[WIND ? NP1 : 1];
+    if constexpr (WIND) {
       f2 xo[NP];
-      swap(cw, xo);
+      swap(ev, xo);
       float pd[2 * NP1];
 #pragma unroll
-      for (int t = 0; t < 2 * NP1; ++t) pd[t] = t < NH1 ? derivative(cw, xo, a, t) : 0.0f;
+      for (int t = 0; t < 2 * NP1; ++t) pd[t] = t < NH1 ? derivative(ev, xo, a, t) : 0.0f;
       __syncwarp();  // keeps the products of the two derivatives apart (registers)
 #pragma unroll
       for (int t = 0; t < NH1; ++t) {
@@ -224,10 +237,12 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
 #pragma unroll
     for (int j = 0; j < NP; ++j) r[j] = f2_zero();
     // two points per pass (an odd last point is paired with itself at weight 0)
-    // Separate wind, many points: the test sums run in blocks of points whose partial sums meet
-    // in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
-    // more than the warp-per-element kernel, whose points are summed pairwise.
-    constexpr int QB = (WSEP && NQ > 64) ? (NQ / 8 + 1) * 2 : NQ;
+    // Separate wind and VJP, many points: the test sums run in blocks of points whose partial sums
+    // meet in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
+    // more than a warp per element, whose points are summed pairwise; one over 46 points rounded
+    // the wind's cotangent 20 % more (at k = 3 the blocks cost 5 us of 61).
+    constexpr int QLIM = MODE == kVolWind ? 64 : (MODE == kVolAdjSame ? 100 : 16);
+    constexpr int QB = (MODE != kVolSame && NQ > QLIM) ? (NQ / 8 + 1) * 2 : NQ;
     float* yp = sY + ((act ? el : 0) * D + a) * NB + h;  // this lane's output entries
 #pragma unroll 1
     for (int q0 = 0; q0 < NQ; q0 += QB) {
@@ -252,9 +267,11 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
 #pragma unroll
             for (int w = 0; w < 2; ++w) {
               const int j = t4 / 2 + w, jc = j < NP ? j : 0, j1 = j < NP1 ? j : 0;
-              if (j < NP) us[x] = f2_fma(p[w], c[jc], us[x]);
-              if constexpr (WSEP) {
-                if (j < NP) ws[x] = f2_fma(p[w], cw[jc], ws[x]);
+              if (!ADJ && j < NP) us[x] = f2_fma(p[w], c[jc], us[x]);
+              if constexpr (MODE != kVolSame) {
+                if (j < NP) ws[x] = f2_fma(p[w], ev[jc], ws[x]);
+              }
+              if constexpr (WIND) {
                 if (j < NP1) ds[x] = f2_fma(p[w], dw[j1], ds[x]);
               }
               if (j < NP1) {
@@ -265,32 +282,45 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
           }
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
-          const float u = halves(f2_sum(us[x]));
+          const float u = ADJ ? 0.0f : halves(f2_sum(us[x]));
           float gd[D];
 #pragma unroll
           for (int cc = 0; cc < D; ++cc) gd[cc] = halves(f2_sum(gs[x][cc]));
-          float f;
-          if constexpr (WSEP) {
-            const float wa = halves(f2_sum(ws[x]));
-            f = halves(f2_sum(ds[x])) * u;
+          const float wa = MODE == kVolSame ? u : halves(f2_sum(ws[x]));
+          float f = 0.0f;
+          if constexpr (ROW) {  // (div^ W) u_a + W . grad^ u_a, or - W . grad^ z_a
+            if (WIND) f = halves(f2_sum(ds[x])) * u;
 #pragma unroll
             for (int cc = 0; cc < D; ++cc) f = fmaf(__shfl_sync(kFull, wa, el * LPE + 2 * cc), gd[cc], f);
-          } else {
-            const float u1 = __shfl_sync(kFull, u, p1);
-            const float u2 = D == 3 ? __shfl_sync(kFull, u, p2) : 0.0f;
+          }
+          if constexpr (MODE == kVolSame) {
             float pd = 0.0f;
 #pragma unroll
             for (int cc = 0; cc < D; ++cc) pd = fmaf(M0[cc], gd[cc], pd);
             float dv = pd + __shfl_sync(kFull, pd, p1);
             if (D == 3) dv += __shfl_sync(kFull, pd, p2);
             f = dv * u;
+          }
+          if constexpr (COLS) {  // W = M u with the other components' u
+            const float u1 = __shfl_sync(kFull, wa, p1);
+            const float u2 = D == 3 ? __shfl_sync(kFull, wa, p2) : 0.0f;
 #pragma unroll
             for (int cc = 0; cc < D; ++cc) {
-              float W = fmaf(M1[cc], u1, M0[cc] * u);
+              float W = fmaf(M1[cc], u1, M0[cc] * wa);
               if (D == 3) W = fmaf(M2[cc], u2, W);
               f = fmaf(W, gd[cc], f);
             }
           }
+          if constexpr (MODE == kVolAdjW || MODE == kVolAdjSame) {  // sum_c M[c][a] sum_b u_b d^_c z_b
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) {
+              const float v = wa * gd[cc];
+              float ug = v + __shfl_sync(kFull, v, p1);
+              if (D == 3) ug += __shfl_sync(kFull, v, p2);
+              f = fmaf(M0[cc], ug, f);
+            }
+          }
+          if (ADJ) f = -f;
           ff[x] = f2_dup(f * (x == 0 || two ? sWq[qs[x]] : 0.0f));
         }
 #pragma unroll
@@ -323,7 +353,8 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
       for (int f = 0; f <= D; ++f) {
 #pragma unroll
         for (int mm = 0; mm < NF; ++mm) {
-          const f2 gv = f2_dup(gl[(f * NF + mm) * D]);
+          const f2 gv = f2_dup(MODE == kVolAdjSame ? gl[(f * NF + mm) * D] + gl[C::GW + (f * NF + mm) * D]
+                                                 : gl[(f * NF + mm) * D]);
           const int i0 = cnbasis(D, mode_degree(D - 1, mm) - 1);  // lower degrees have no such trace
           const float* trow = sTrM + (f * NF + mm) * RW + h * HP;
 #pragma unroll
@@ -351,8 +382,8 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, WSEP>::WARPS, VolRH<D, K, WSE
     if (act) {
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
-        if (2 * j < nh) yp[4 * j] = f2_x(r[j]) * invabs;
-        if (2 * j + 1 < nh) yp[4 * j + 2] = f2_y(r[j]) * invabs;
+        if (2 * j < nh) yp[4 * j] = f2_x(r[j]) * (ADJ ? 1.0f : invabs);
+        if (2 * j + 1 < nh) yp[4 * j + 2] = f2_y(r[j]) * (ADJ ? 1.0f : invabs);
       }
     }
     __syncwarp();

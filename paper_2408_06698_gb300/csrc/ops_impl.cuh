@@ -11,7 +11,6 @@
 #include "kernels_adapt.cuh"
 #include "kernels_vr.cuh"
 #include "kernels_vrh.cuh"
-#include "kernels_var.cuh"
 #include "kernels_far.cuh"
 #include "kernels_fr.cuh"
 
@@ -98,15 +97,37 @@ class OpsImpl final : public Ops {
   static_assert(!std::is_same<T, float>::value || kVolR || kVolRH, "a register volume kernel for every FP32 order");
   int g_volrh_ = 1;
   // separate wind in FP32: the register kernel, its half-basis form where a lane's registers run out
-  static constexpr bool kVolRW = std::is_same<T, float>::value && VolR<D, K, false, true>::OK;
+  static constexpr bool kVolRW = std::is_same<T, float>::value && VolR<D, K, false, kVolWind>::OK;
   static constexpr bool kVolRHW = std::is_same<T, float>::value && !kVolRW;
   int g_volw_ = 1;
-  // register-resident adjoint volume kernel (w = u)
-  static constexpr bool kVolAR = std::is_same<T, float>::value && VolAR<D, K>::OK;
-  int g_volar_ = 1;
-  // register-resident adjoint facet kernel (w = u)
-  static constexpr bool kFacAR = std::is_same<T, float>::value && FacAR<D, K>::OK;
-  int g_facar_ = 1;
+  // volume part of the VJP in FP32: the register kernel of each cotangent (kVolAdjU, kVolAdjW,
+  // kVolAdjSame), its half-basis form where a lane's registers run out
+  static constexpr bool kVolAdjR = VolR<D, K, false, kVolAdjSame>::OK;
+  int g_volar_[3] = {1, 1, 1};
+  template <int MODE>
+  using VolA = typename std::conditional<kVolAdjR, VolR<D, K, false, MODE>, VolRH<D, K, MODE>>::type;
+  template <int MODE>
+  cudaError_t setup_adj() {
+    using R = VolA<MODE>;
+    static_assert(R::OK, "a register kernel for every FP32 order");
+    if constexpr (kVolAdjR) return setup(k_volume_r<D, K, false, false, MODE>, R::SMEM, 32 * R::WARPS, &g_volar_[MODE - kVolAdjU]);
+    else return setup(k_volume_rh<D, K, MODE>, R::SMEM, 32 * R::WARPS, &g_volar_[MODE - kVolAdjU]);
+  }
+  template <int MODE>
+  void launch_adj(const DevMesh& m, const DevTabs& t, const void* in1, const void* ybar, const void* gam,
+                  const void* gam2, void* out, cudaStream_t st) {
+    using R = VolA<MODE>;
+    const int g = clamp_grid(g_volar_[MODE - kVolAdjU], (m.E + R::ELW - 1) / R::ELW, 1);
+    if constexpr (kVolAdjR)
+      launch(k_volume_r<D, K, false, false, MODE>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(in1),
+             static_cast<const float*>(ybar), static_cast<const float*>(gam), static_cast<const float*>(gam2),
+             static_cast<float*>(out), Combine(), static_cast<float*>(nullptr));
+    else
+      launch(k_volume_rh<D, K, MODE>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(in1),
+             static_cast<const float*>(ybar), static_cast<const float*>(gam), static_cast<const float*>(gam2),
+             static_cast<float*>(out), Combine());
+  }
+  int g_facar_[2] = {1, 1};  // facet part of the VJP in FP32: w = u, separate wind
   int g_volr_ = 1, g_volrf_ = 1;
   // facet term: register-resident kernel in FP32 (every order), a warp per facet in FP64
   static constexpr bool kFacR = std::is_same<T, float>::value;
@@ -231,10 +252,19 @@ class OpsImpl final : public Ops {
       }
     }
     if ((err = setup(k_eta<D, K, T>, eta_smem(), th, &g_eta_)) != cudaSuccess) return err;
-    if ((err = setup(k_facet_adj<D, K, T, false>, facet_adj_smem(false), th, &g_fadj_)) != cudaSuccess) return err;
-    if ((err = setup(k_facet_adj<D, K, T, true>, facet_adj_smem(true), th, &g_fadj_)) != cudaSuccess) return err;
-    if ((err = setup(k_volume_adj<D, K, T, false>, volume_adj_smem(false), th, &g_vadj_)) != cudaSuccess) return err;
-    if ((err = setup(k_volume_adj<D, K, T, true>, volume_adj_smem(true), th, &g_vadj_)) != cudaSuccess) return err;
+    if constexpr (std::is_same<T, float>::value) {
+      using R = FacR<D, K>;
+      if ((err = setup(k_facet_adj_r<D, K, false>, R::SMEM, 32 * R::WARPS, &g_facar_[0])) != cudaSuccess) return err;
+      if ((err = setup(k_facet_adj_r<D, K, true>, R::SMEM, 32 * R::WARPS, &g_facar_[1])) != cudaSuccess) return err;
+      if ((err = setup_adj<kVolAdjU>()) != cudaSuccess) return err;
+      if ((err = setup_adj<kVolAdjW>()) != cudaSuccess) return err;
+      if ((err = setup_adj<kVolAdjSame>()) != cudaSuccess) return err;
+    } else {
+      if ((err = setup(k_facet_adj<D, K, T, false>, facet_adj_smem(false), th, &g_fadj_)) != cudaSuccess) return err;
+      if ((err = setup(k_facet_adj<D, K, T, true>, facet_adj_smem(true), th, &g_fadj_)) != cudaSuccess) return err;
+      if ((err = setup(k_volume_adj<D, K, T, false>, volume_adj_smem(false), th, &g_vadj_)) != cudaSuccess) return err;
+      if ((err = setup(k_volume_adj<D, K, T, true>, volume_adj_smem(true), th, &g_vadj_)) != cudaSuccess) return err;
+    }
     if constexpr (kFacR) {
       using R = FacR<D, K>;
       if ((err = setup(k_facet_r<D, K, false>, R::SMEM, 32 * R::WARPS, &g_facr_[0])) != cudaSuccess) return err;
@@ -249,36 +279,28 @@ class OpsImpl final : public Ops {
     }
     if ((err = setup(k_volume<D, K, T, true, kVolumeTab, false>, volume_smem(true), th, &g_vol_[1])) != cudaSuccess) return err;
     if constexpr (kVolR) {
-      if ((err = setup(k_volume_r<D, K, false, false, false>, VolR<D, K>::SMEM, 32 * VolR<D, K>::WARPS, &g_volr_)) != cudaSuccess)
-        return err;
-    }
-    if constexpr (kFacAR) {
-      if ((err = setup(k_facet_adj_r<D, K>, FacAR<D, K>::SMEM, 32 * FacAR<D, K>::WARPS, &g_facar_)) != cudaSuccess)
-        return err;
-    }
-    if constexpr (kVolAR) {
-      if ((err = setup(k_volume_adj_r<D, K>, VolAR<D, K>::SMEM, 32 * VolAR<D, K>::WARPS, &g_volar_)) != cudaSuccess)
+      if ((err = setup(k_volume_r<D, K, false, false, kVolSame>, VolR<D, K>::SMEM, 32 * VolR<D, K>::WARPS, &g_volr_)) != cudaSuccess)
         return err;
     }
     if constexpr (kVolRH) {
-      if ((err = setup(k_volume_rh<D, K, false>, VolRH<D, K>::SMEM, 32 * VolRH<D, K>::WARPS, &g_volrh_)) != cudaSuccess)
+      if ((err = setup(k_volume_rh<D, K, kVolSame>, VolRH<D, K>::SMEM, 32 * VolRH<D, K>::WARPS, &g_volrh_)) != cudaSuccess)
         return err;
     }
     if constexpr (kVolRW) {
-      using R = VolR<D, K, false, true>;
-      if ((err = setup(k_volume_r<D, K, false, false, true>, R::SMEM, 32 * R::WARPS, &g_volw_)) != cudaSuccess) return err;
+      using R = VolR<D, K, false, kVolWind>;
+      if ((err = setup(k_volume_r<D, K, false, false, kVolWind>, R::SMEM, 32 * R::WARPS, &g_volw_)) != cudaSuccess) return err;
     }
     if constexpr (kVolRHW) {
-      using R = VolRH<D, K, true>;
-      if ((err = setup(k_volume_rh<D, K, true>, R::SMEM, 32 * R::WARPS, &g_volw_)) != cudaSuccess) return err;
+      using R = VolRH<D, K, kVolWind>;
+      if ((err = setup(k_volume_rh<D, K, kVolWind>, R::SMEM, 32 * R::WARPS, &g_volw_)) != cudaSuccess) return err;
     }
     if constexpr (kVolRT) {
-      if ((err = setup(k_volume_r<D, K, false, true, false>, VolR<D, K, true>::SMEM, 32 * VolR<D, K, true>::WARPS,
+      if ((err = setup(k_volume_r<D, K, false, true, kVolSame>, VolR<D, K, true>::SMEM, 32 * VolR<D, K, true>::WARPS,
                        &g_volrt_)) != cudaSuccess)
         return err;
     }
     if constexpr (kVolRF) {
-      if ((err = setup(k_volume_r<D, K, true, false, false>, VolR<D, K>::SMEM_FUSE, 32 * VolR<D, K>::WARPS, &g_volrf_)) !=
+      if ((err = setup(k_volume_r<D, K, true, false, kVolSame>, VolR<D, K>::SMEM_FUSE, 32 * VolR<D, K>::WARPS, &g_volrf_)) !=
           cudaSuccess)
         return err;
     }
@@ -380,8 +402,8 @@ class OpsImpl final : public Ops {
       if (!wsep && (vvar_ == kVolRegHalf || !kVolR)) {
         using R = VolRH<D, K>;
         const int g = clamp_grid(g_volrh_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_rh<D, K, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(out), c);
+        launch(k_volume_rh<D, K, kVolSame>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<const float*>(nullptr), static_cast<float*>(out), c);
         return 1;
       }
     }
@@ -389,8 +411,8 @@ class OpsImpl final : public Ops {
       if (!wsep && vvar_ == kVolRegTab) {
         using R = VolR<D, K, true>;
         const int g = clamp_grid(g_volrt_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_r<D, K, false, true, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
+        launch(k_volume_r<D, K, false, true, kVolSame>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<const float*>(nullptr), static_cast<float*>(out), c, static_cast<float*>(nullptr));
         return 1;
       }
     }
@@ -398,8 +420,8 @@ class OpsImpl final : public Ops {
       if (!wsep) {
         using R = VolR<D, K>;
         const int g = clamp_grid(g_volr_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_r<D, K, false, false, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
+        launch(k_volume_r<D, K, false, false, kVolSame>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<const float*>(nullptr), static_cast<float*>(out), c, static_cast<float*>(nullptr));
         return 1;
       }
     }
@@ -411,15 +433,15 @@ class OpsImpl final : public Ops {
     if constexpr (kVolRW || kVolRHW) {
       if (m.E > (int64_t)g_vol_[1] * kWarps) {
         if constexpr (kVolRW) {
-          using R = VolR<D, K, false, true>;
-          launch(k_volume_r<D, K, false, false, true>, clamp_grid(g_volw_, (m.E + R::ELW - 1) / R::ELW, 1),
+          using R = VolR<D, K, false, kVolWind>;
+          launch(k_volume_r<D, K, false, false, kVolWind>, clamp_grid(g_volw_, (m.E + R::ELW - 1) / R::ELW, 1),
                  32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL), static_cast<const float*>(wL),
-                 static_cast<const float*>(gam), static_cast<float*>(out), c, static_cast<float*>(nullptr));
+                 static_cast<const float*>(gam), static_cast<const float*>(nullptr), static_cast<float*>(out), c, static_cast<float*>(nullptr));
         } else {
-          using R = VolRH<D, K, true>;
-          launch(k_volume_rh<D, K, true>, clamp_grid(g_volw_, (m.E + R::ELW - 1) / R::ELW, 1), 32 * R::WARPS, R::SMEM,
+          using R = VolRH<D, K, kVolWind>;
+          launch(k_volume_rh<D, K, kVolWind>, clamp_grid(g_volw_, (m.E + R::ELW - 1) / R::ELW, 1), 32 * R::WARPS, R::SMEM,
                  st, m, t, static_cast<const float*>(uL), static_cast<const float*>(wL),
-                 static_cast<const float*>(gam), static_cast<float*>(out), c);
+                 static_cast<const float*>(gam), static_cast<const float*>(nullptr), static_cast<float*>(out), c);
         }
         return 1;
       }
@@ -460,50 +482,54 @@ class OpsImpl final : public Ops {
   int facet_adj(const DevMesh& m, const DevTabs& t, const void* uL, const void* wL, const void* ybar, int l,
                 const int8_t* facet_l, void* gamU, void* gamW, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
-    if constexpr (kFacAR) {
-      if (!wsep) {
-        using R = FacAR<D, K>;
-        const int g = clamp_grid(g_facar_, (m.NF + R::FPW - 1) / R::FPW, 1);
-        launch(k_facet_adj_r<D, K>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(ybar), l, facet_l, static_cast<float*>(gamU), static_cast<float*>(gamW));
-        return 1;
-      }
+    if constexpr (std::is_same<T, float>::value) {
+      using R = FacR<D, K>;
+      const int g = clamp_grid(g_facar_[wsep ? 1 : 0], (m.NF + R::FPW - 1) / R::FPW, 1);
+      if (wsep)
+        launch(k_facet_adj_r<D, K, true>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(wL), static_cast<const float*>(ybar), l, facet_l, static_cast<float*>(gamU),
+               static_cast<float*>(gamW));
+      else
+        launch(k_facet_adj_r<D, K, false>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(ybar), l, facet_l, static_cast<float*>(gamU),
+               static_cast<float*>(gamW));
+    } else {
+      const int g = clamp_grid(g_fadj_, m.NF, kWarps);
+      if (wsep)
+        launch(k_facet_adj<D, K, T, true>, g, 32 * kWarps, facet_adj_smem(true), st,
+            m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar), l, facet_l,
+            static_cast<T*>(gamU), static_cast<T*>(gamW));
+      else
+        launch(k_facet_adj<D, K, T, false>, g, 32 * kWarps, facet_adj_smem(false), st,
+            m, t, static_cast<const T*>(uL), static_cast<const T*>(uL), static_cast<const T*>(ybar), l, facet_l,
+            static_cast<T*>(gamU), static_cast<T*>(gamW));
     }
-    const int g = clamp_grid(g_fadj_, m.NF, kWarps);
-    if (wsep)
-      launch(k_facet_adj<D, K, T, true>, g, 32 * kWarps, facet_adj_smem(true), st, 
-          m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar), l, facet_l,
-          static_cast<T*>(gamU), static_cast<T*>(gamW));
-    else
-      launch(k_facet_adj<D, K, T, false>, g, 32 * kWarps, facet_adj_smem(false), st, 
-          m, t, static_cast<const T*>(uL), static_cast<const T*>(uL), static_cast<const T*>(ybar), l, facet_l,
-          static_cast<T*>(gamU), static_cast<T*>(gamW));
     return 1;
   }
 
   int volume_adj(const DevMesh& m, const DevTabs& t, const void* uL, const void* wL, const void* ybar,
                  const void* gamU, const void* gamW, void* ubar, void* wbar, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
-    if constexpr (kVolAR) {
+    if constexpr (std::is_same<T, float>::value) {
       if (!wsep) {
-        using R = VolAR<D, K>;
-        const int g = clamp_grid(g_volar_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_adj_r<D, K>, g, 32 * R::WARPS, R::SMEM, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(ybar), static_cast<const float*>(gamU), static_cast<const float*>(gamW),
-               static_cast<float*>(ubar));
+        launch_adj<kVolAdjSame>(m, t, uL, ybar, gamU, gamW, ubar, st);
         return 1;
       }
+      if (ubar) launch_adj<kVolAdjU>(m, t, wL, ybar, gamU, nullptr, ubar, st);
+      if (wbar) launch_adj<kVolAdjW>(m, t, uL, ybar, gamW, nullptr, wbar, st);
+      return (ubar != nullptr) + (wbar != nullptr);
+    } else {
+      const int g = clamp_grid(g_vadj_, m.E, kWarps);
+      if (wsep)
+        launch(k_volume_adj<D, K, T, true>, g, 32 * kWarps, volume_adj_smem(true), st,
+            m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar),
+            static_cast<const T*>(gamU), static_cast<const T*>(gamW), static_cast<T*>(ubar), static_cast<T*>(wbar));
+      else
+        launch(k_volume_adj<D, K, T, false>, g, 32 * kWarps, volume_adj_smem(false), st,
+            m, t, static_cast<const T*>(uL), static_cast<const T*>(uL), static_cast<const T*>(ybar),
+            static_cast<const T*>(gamU), static_cast<const T*>(gamW), static_cast<T*>(ubar), static_cast<T*>(nullptr));
+      return 1;
     }
-    const int g = clamp_grid(g_vadj_, m.E, kWarps);
-    if (wsep)
-      launch(k_volume_adj<D, K, T, true>, g, 32 * kWarps, volume_adj_smem(true), st, 
-          m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar),
-          static_cast<const T*>(gamU), static_cast<const T*>(gamW), static_cast<T*>(ubar), static_cast<T*>(wbar));
-    else
-      launch(k_volume_adj<D, K, T, false>, g, 32 * kWarps, volume_adj_smem(false), st, 
-          m, t, static_cast<const T*>(uL), static_cast<const T*>(uL), static_cast<const T*>(ybar),
-          static_cast<const T*>(gamU), static_cast<const T*>(gamW), static_cast<T*>(ubar), nullptr);
-    return 1;
   }
 
   int volume_l2v(const DevMesh& m, const DevTabs& t, const void* uL, const void* gam, void* lf, Combine c,
@@ -523,8 +549,8 @@ class OpsImpl final : public Ops {
       if (vvar_ == kVolRegFused) {
         using R = VolR<D, K>;
         const int g = clamp_grid(g_volrf_, (m.E + R::ELW - 1) / R::ELW, 1);
-        launch(k_volume_r<D, K, true, false, false>, g, 32 * R::WARPS, R::SMEM_FUSE, st, m, t, static_cast<const float*>(uL),
-               static_cast<const float*>(uL), static_cast<const float*>(gam), static_cast<float*>(outV), c, static_cast<float*>(lf));
+        launch(k_volume_r<D, K, true, false, kVolSame>, g, 32 * R::WARPS, R::SMEM_FUSE, st, m, t, static_cast<const float*>(uL),
+               static_cast<const float*>(uL), static_cast<const float*>(gam), nullptr, static_cast<float*>(outV), c, static_cast<float*>(lf));
         return 1;
       }
     }

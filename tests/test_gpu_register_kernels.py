@@ -10,6 +10,7 @@ import pytest
 import torch
 
 import workloads as W
+from oracle import adjoint as A
 from oracle import convection as C
 from oracle import fe, hdiv, mesh
 
@@ -78,3 +79,20 @@ def test_apply_every_order(dim, n, k, walls):
         g.set_facet_l(torch.as_tensor(fl, device=g.device))
         y = apply()
         assert _rel(y, C.apply(topo, ref, wind, u, fl.astype(np.int64), exterior=exterior, inlet=inlet)) < 1e-6
+
+
+@pytest.mark.parametrize("dim,n,k", ORDERS)
+def test_vjp_per_facet_orders(dim, n, k):
+    """The VJP kernels with an order per facet; tolerance of the FP32 VJP parity tests, 2e-6."""
+    g, topo, ref = _setup(dim, n, k, False)
+    sp = hdiv.HDiv(topo, ref)
+    rng = np.random.default_rng(7700 + 10 * dim + k)
+    shape = (topo.n_elems, dim, ref.nb)
+    wV, u, yb = (rng.standard_normal(s).astype(np.float32).astype(np.float64) for s in (sp.n_hdiv, shape, shape))
+    fl = rng.integers(-1, k + 1, size=topo.n_facets).astype(np.int8)
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x).reshape(-1), dtype=torch.float32, device=g.device)  # noqa: E731
+    g.set_facet_l(torch.as_tensor(fl, device=g.device))
+    wbar, ubar = g.vjp_apply(dev(wV), dev(u), dev(yb))
+    wb, ub = A.vjp_apply(topo, ref, sp.to_l2(wV), u, yb, fl.astype(np.int64))
+    assert _rel(ubar, ub) < 2e-6
+    assert _rel(wbar, sp.dual(wb)) < 2e-6
