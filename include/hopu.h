@@ -97,7 +97,9 @@ typedef enum {
                         them faster: the two dense products of the refined V_h -> L2
                         projection (its residual stays compensated FP32 on the CUDA cores,
                         so the projection keeps the accuracy of HOPU_FP32), the element part
-                        of the back-projection, and the STAGE volume contractions (3D k <= 3)
+                        of the back-projection, and the STAGE volume contractions (3D k <= 3; 3D
+                        k = 3, 4 also with three BF16 parts per operand and six products, an
+                        error below FP32 rounding)
                                                                                             */
   HOPU_TF32 = 3      /* FP32 coefficients; the V_h -> L2 projection GEMM, the back-projection
                         and the STAGE volume contractions on the tensor cores with one TF32
@@ -170,10 +172,13 @@ hopu_status hopu_tuning(const hopu_ctx* ctx, int* out2);
  *       registers, more resident warps) + the separate back-projection,
  *   5 = register-resident kernel with each (element, component)'s basis split over two
  *       lanes (half the registers per lane; FP32 k <= 5) + the separate back-projection,
+ *   6 = tensor-core kernel with the elements along the MMA rows (HOPU_FP32_TC, 3D k = 3, 4;
+ *       operands in three BF16 parts) + the separate back-projection,
  *  -1 = warp-per-element kernel and the separate back-projection (no other variant for
  *       this order and precision).
  * ms6 (host, 6 doubles, may be NULL): the autotuner's time per launch of each variant on
- * this mesh in ms, -1 for variants not timed (one variant only, or not available).  No
+ * this mesh in ms for variants 0 .. 5, -1 for those not timed (one variant only, or not
+ * available).  No
  * paper counterpart (launch tuning).                                                  */
 hopu_status hopu_tuning_volume(const hopu_ctx* ctx, int* variant, double* ms6);
 

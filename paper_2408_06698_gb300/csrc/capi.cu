@@ -298,8 +298,8 @@ hopu_status device_status(hopu_ctx* c) {
 void free_all(hopu_ctx* c) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
-  void* ptrs[] = {c->d_elog_pos, c->d_mesh, c->d_geoT, c->d_tabs, c->d_gam, c->d_lf, c->d_uL, c->d_yL, c->d_wL,
-                  c->d_wfz, c->d_s1, c->d_s2, c->d_diss, c->d_red, c->d_gamW, c->d_adj, c->d_err, c->d_tcvol,
+  void* ptrs[] = {c->d_elog_pos, c->d_mesh, c->d_geoT, c->d_geoF, c->d_tabs, c->d_gam, c->d_lf, c->d_uL, c->d_yL, c->d_wL,
+                  c->d_wfz, c->d_s1, c->d_s2, c->d_diss, c->d_red, c->d_gamW, c->d_adj, c->d_err, c->d_tcvol, c->d_tcvole,
                   c->d_inlet, c->d_inlet_modes, c->d_csr, c->d_tcl2v, c->d_tcv2l, c->d_csr_tc};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -539,6 +539,52 @@ void tensor_core_volume_table(const RefTables& R, std::vector<float>& out) {
     }
 }
 
+// Round to BF16 (round to nearest even), as the bits of its upper half.
+uint16_t bf16_round(double x, double* back) {
+  const float f = (float)x;
+  uint32_t u;
+  std::memcpy(&u, &f, 4);
+  u = (u + 0x7fffu + ((u >> 16) & 1u)) & 0xffff0000u;
+  float r;
+  std::memcpy(&r, &u, 4);
+  *back = (double)r;
+  return (uint16_t)(u >> 16);
+}
+
+// B operands of the tensor-core volume kernel with elements along the rows: B1 with rows (half of
+// the points, field f, point) = phi_i(x_q) (f = 0) and d phi_i / d xhat_{f-1}(x_q), then B2[i][q] =
+// phi_i(x_q) and B3[i][f nf + m] = TrM[f][m][i] (parts stacked by rows, NS rows each, then 8 zero
+// rows, and part 0 of B3 once more), each in three BF16 parts (their sum carries 24 bits), blocked K-major: core matrices of 8 rows x 8 values, 128
+// bytes each; zero outside the points and the basis.  Bt, dBt: the tables of kernel_tables (rows of
+// nbq).
+void tensor_core_volume_el_table(const RefTables& R, const std::vector<double>& Bt, const std::vector<double>& dBt,
+                                 int nbq, std::vector<uint16_t>& out) {
+  const int nb = R.nb, nq = R.nqk, NQP = vol_te_nqp(nq), KP = vol_te_kp(nb), KF = vol_te_kf(nq), NS = vol_te_ns(nb);
+  const int P0 = vol_te_p0(nq), nfm = (R.dim + 1) * R.nf, KG = vol_te_kg(nfm);
+  const size_t P1 = (size_t)4 * NQP * KP, O2 = 3 * P1, O3 = O2 + (size_t)(3 * NS + 8) * KF;
+  out.assign(O3 + (size_t)(4 * NS + 8) * KG, 0);
+  // the parts of v at element (row, col) of the operand at base, part x `part` values further
+  auto put = [&](size_t base, size_t part, int row, int col, int kp, double v) {
+    const size_t o = base + ((size_t)(row >> 3) * (kp >> 3) + (col >> 3)) * 64 + (row & 7) * 8 + (col & 7);
+    for (int x = 0; x < 3; ++x) {
+      double b;
+      out[o + x * part] = bf16_round(v, &b);
+      v -= b;
+    }
+  };
+  for (int q = 0; q < nq; ++q)
+    for (int i = 0; i < nb; ++i) {
+      const double v = Bt[(size_t)q * nbq + i];
+      const int np = q < P0 ? P0 : NQP - P0, row = q < P0 ? q : 4 * P0 + q - P0;
+      put(0, P1, row, i, KP, v);
+      for (int c = 0; c < 3; ++c) put(0, P1, row + (c + 1) * np, i, KP, dBt[((size_t)c * nq + q) * nbq + i]);
+      put(O2, (size_t)NS * KF, i, q, KF, v);
+    }
+  for (int f = 0; f < nfm; ++f)
+    for (int i = 0; i < nb; ++i) put(O3, (size_t)NS * KG, i, f, KG, R.trm[(size_t)f * nb + i]);
+  std::copy_n(out.begin() + O3, (size_t)NS * KG, out.begin() + O3 + (size_t)(3 * NS + 8) * KG);
+}
+
 // B operand of the tensor-core back-projection: B[r][kappa(b, i)] = D[r][b nb + i] (r the
 // local functional, b the component, i the basis index, kappa the K column of l2v_tc_gw),
 // N = nloc padded to 16 rows; hi = tf32(D), lo = tf32(D - hi), the hi parts then the lo
@@ -771,7 +817,7 @@ hopu_status autotune(hopu_ctx* c, int hint) {
   std::vector<int> cand;
   for (int v = 0; v < kVolVariants; ++v) {
     if (!o->volume_variant_ok(v)) continue;
-    if (hint == 1 && v == kVolTensor) continue;
+    if (hint == 1 && (v == kVolTensor || v == kVolTensorEl)) continue;
     if (hint == 2 && o->volume_variant_ok(kVolTensor) && v != kVolTensor) continue;
     cand.push_back(v);
   }
@@ -923,6 +969,14 @@ hopu_status create_impl(const hopu_mesh_desc* mesh, const hopu_options* opts, vo
     HOPU_CUDA(c, cudaMalloc(&c->d_geoT, sizeof(double) * gt.size()));
     HOPU_CUDA(c, cudaMemcpy(c->d_geoT, gt.data(), sizeof(double) * gt.size(), cudaMemcpyHostToDevice));
     c->dm.geoT = static_cast<const double*>(c->d_geoT);
+    if (!c->fp64) {  // the same factors and the facet geometry rounded once (what a load and a rounding give)
+      std::vector<float> gf(gt.begin(), gt.end());
+      gf.insert(gf.end(), c->topo.fgeo.begin(), c->topo.fgeo.end());
+      HOPU_CUDA(c, cudaMalloc(&c->d_geoF, sizeof(float) * gf.size()));
+      HOPU_CUDA(c, cudaMemcpy(c->d_geoF, gf.data(), sizeof(float) * gf.size(), cudaMemcpyHostToDevice));
+      c->dm.geoF = static_cast<const float*>(c->d_geoF);
+      c->dm.fgeoF = c->dm.geoF + gt.size();
+    }
   }
 
   // tables upload, converted to the working precision
@@ -961,6 +1015,13 @@ hopu_status create_impl(const hopu_mesh_desc* mesh, const hopu_options* opts, vo
     HOPU_CUDA(c, cudaMalloc(&c->d_tcvol, tv.size() * sizeof(float)));
     HOPU_CUDA(c, cudaMemcpy(c->d_tcvol, tv.data(), tv.size() * sizeof(float), cudaMemcpyHostToDevice));
     c->dt.tcvol = c->d_tcvol;
+  }
+  if (c->ops->tensor_core_volume_el()) {
+    std::vector<uint16_t> tv;
+    tensor_core_volume_el_table(R, tabs[0], tabs[13], point_row_stride(R.nb, c->fp64), tv);
+    HOPU_CUDA(c, cudaMalloc(&c->d_tcvole, tv.size() * sizeof(uint16_t)));
+    HOPU_CUDA(c, cudaMemcpy(c->d_tcvole, tv.data(), tv.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
+    c->dt.tcvole = c->d_tcvole;
   }
   if (c->ops->tensor_cores() && c->prec == HOPU_FP32_TC) {
     std::vector<float> csr;
@@ -1085,7 +1146,7 @@ hopu_status hopu_tuning_volume(const hopu_ctx* c, int* variant, double* ms6) {
   if (!c || !variant) return HOPU_EINVAL;
   *variant = c->ops ? c->ops->volume_variant() : -1;
   if (ms6)
-    for (int v = 0; v < kVolVariants; ++v) ms6[v] = c->vol_ms[v];
+    for (int v = 0; v < kVolTimed; ++v) ms6[v] = c->vol_ms[v];
   return HOPU_OK;
 }
 

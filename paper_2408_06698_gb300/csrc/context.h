@@ -29,12 +29,14 @@ struct hopu_ctx {
   Ops* ops = nullptr;
   int nsm = 1, red_blocks = 1;
   double l2v_ms[2] = {-1.0, -1.0};  // autotuner: ms per launch of the FMA / tensor-core back-projection
-  double vol_ms[6] = {-1.0, -1.0, -1.0, -1.0, -1.0, -1.0};  // autotuner: ms per launch of each STAGE volume variant
+  double vol_ms[hopu::kVolVariants] = {-1.0, -1.0, -1.0, -1.0, -1.0, -1.0, -1.0};  // autotuner: ms per launch of each STAGE volume variant
   // device memory
   void* d_mesh = nullptr;   // geo, efc, fa, fb, fgeo
+  void* d_geoF = nullptr;   // FP32: geometry factors rounded to FP32 (DevMesh::geoF, fgeoF)
   void* d_geoT = nullptr;   // working-precision geometry factors
   void* d_tabs = nullptr;   // every reference table
   void* d_tcvol = nullptr;  // tensor-core volume tables (FP32 tensor-core modes)
+  void* d_tcvole = nullptr; // tables of the tensor-core volume kernel with elements along the rows
   void* d_tcv2l = nullptr;  // tensor-core refined projection table (HOPU_FP32_TC)
   void* d_csr_tc = nullptr; // its CSR of D with grouped rows
   void* d_tcl2v = nullptr;  // tensor-core back-projection table (FP32 tensor-core modes)

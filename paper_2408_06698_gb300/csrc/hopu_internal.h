@@ -14,6 +14,9 @@ struct DevMesh {
   const double* geoT = nullptr;  // [E][geoT_stride(d)] FP64 in every precision mode (the FP32 kernels
                                  // round each factor when they load it):
                                  //   Pf = J / det J, Pi = det J * Jinv, M = |det J| * Jinv, 1/|det J|
+  const float* geoF = nullptr;   // FP32 contexts: geoT and fgeo rounded to FP32, same layouts.  A conversion
+  const float* fgeoF = nullptr;  // at the load runs on the FP64 unit: ten per thread were 3200 cycles of a
+                                 // 40-element tile of k_volume_te
   const int32_t* efc = nullptr;  // [E][d+1]: F*4 + (sigma<0)*2 + (element is side B)
   const int32_t* fa = nullptr;   // [NF]: element*4 + local facet of side A
   const int32_t* fb = nullptr;   // [NF]: same for side B
@@ -58,6 +61,8 @@ struct DevTabs {
                                 //                 multiple of 16 bytes), zero padding
   const void* tcv2l = nullptr;  // FP32 3xTF32 refined projection table (Dinv as the B operand,
                                 //   TF32 hi and lo parts, layout of V2lTcr), or NULL
+  const void* tcvole = nullptr; // tables of k_volume_te (FP32_TC, 3D k = 3, 4): the B operands in three
+                                //   BF16 parts each, or NULL
   const void* tcl2v = nullptr;  // FP32 tensor-core back-projection table (D as the B operand,
                                 //   TF32 hi and lo parts, layout of L2vTc), or NULL
 };
@@ -100,6 +105,17 @@ inline constexpr int v2l_tc_rpg(int nloc) { return (nloc + 3) / 4; }
 inline constexpr int v2l_tc_gw(int nloc) { return (v2l_tc_rpg(nloc) + 3) / 4 * 4; }
 inline constexpr int v2l_tc_kp(int nloc) { return 4 * v2l_tc_gw(nloc); }
 
+// Sizes of the tensor-core volume kernel with elements along the rows (k_volume_te and its host
+// table): groups of warps, points per field padded to 4, K of the products padded to 16, columns of a
+// block of the second result.
+inline constexpr int vol_te_groups(int nb) { return nb > 24 ? 3 : 2; }
+inline constexpr int vol_te_nqp(int nq) { return (nq + 3) / 4 * 4; }
+inline constexpr int vol_te_kp(int nb) { return (nb + 15) / 16 * 16; }
+inline constexpr int vol_te_kf(int nq) { return (vol_te_nqp(nq) + 15) / 16 * 16; }
+inline constexpr int vol_te_p0(int nq) { return (vol_te_nqp(nq) / 2 + 3) / 4 * 4; }  // points of the first half
+inline constexpr int vol_te_kg(int nfm) { return (nfm + 15) / 16 * 16; }              // K of the facet moments
+inline constexpr int vol_te_ns(int nb) { return (nb + 7) / 8 * 8; }
+
 // layout of the working-precision geometry record (offsets in elements)
 inline constexpr int geoT_stride(int d) { return ((3 * d * d + 1 + 3) / 4) * 4; }
 
@@ -116,7 +132,9 @@ enum VolumeVariant {
   kVolTensor = 3,     // tensor-core kernel
   kVolRegTab = 4,     // register kernel with reference-gradient tables + separate back-projection
   kVolRegHalf = 5,    // register kernel, basis split over two lanes + separate back-projection
-  kVolVariants = 6
+  kVolTimed = 6,      // variants whose times hopu_tuning_volume reports
+  kVolTensorEl = 6,   // tensor-core kernel with elements along the rows + separate back-projection
+  kVolVariants = 7
 };
 
 // One family of kernels for a fixed (dim, k, precision).  Every call enqueues on the
@@ -146,6 +164,7 @@ class Ops {
   virtual bool has_fused() const = 0;
   virtual bool tensor_cores() const = 0;  // the V_h -> L2 projection runs on tensor cores
   virtual bool tensor_core_volume() const = 0;  // a tensor-core fused STAGE volume kernel exists
+  virtual bool tensor_core_volume_el() const = 0;  // ... the one with elements along the rows
   // variant choice per kernel family (autotuner): 0 = FP32 FMA kernel, 1 = tensor-core kernel
   virtual void select(int v2l_tc, int volume_tc) = 0;
   virtual int selected_v2l() const = 0;

@@ -8,6 +8,7 @@
 #include "kernels_adj.cuh"
 #include "kernels_tc.cuh"
 #include "kernels_tcr.cuh"
+#include "kernels_tcv.cuh"
 #include "kernels_adapt.cuh"
 #include "kernels_vr.cuh"
 #include "kernels_vrh.cuh"
@@ -82,6 +83,9 @@ class OpsImpl final : public Ops {
   bool tcr_fits_ = true;  // the CSR of D fits beside the refined tensor-core projection's tiles
   static constexpr bool kTcVol = std::is_same<T, float>::value && VolTc<D, K>::OK;
   int g_vol_tc_ = 1;
+  // tensor-core STAGE volume kernel with elements along the rows (3xBF16 parts: HOPU_FP32_TC only)
+  static constexpr bool kTcVolE = std::is_same<T, float>::value && VolTe<D, K>::OK;
+  int g_vol_te_ = 1;
   static constexpr bool kTcL2v = std::is_same<T, float>::value && L2vTc<D, K>::OK;
   int g_l2v_tc_ = 1;
   bool use_tc_l2v_ = false;  // autotuner choice of the element back-projection
@@ -195,6 +199,7 @@ class OpsImpl final : public Ops {
   // coefficients of smooth fields that a plain FP32 or 3xTF32 product loses.
   bool tensor_cores() const override { return (tc_ == 1 && kTcV2l) || (tc_ == 3 && kTcV2lR && tcr_fits_); }
   bool tensor_core_volume() const override { return tc_ != 0 && kTcVol; }
+  bool tensor_core_volume_el() const override { return tc_ == 3 && kTcVolE; }
   void select(int v2l_tc, int volume_tc) override {
     use_tc_v2l_ = v2l_tc != 0 && tensor_cores();
     if (volume_tc != 0 && tensor_core_volume()) vvar_ = kVolTensor;
@@ -208,6 +213,7 @@ class OpsImpl final : public Ops {
       case kVolRegSplit: return kVolR;
       case kVolWarpFused: return kFuse;
       case kVolTensor: return tensor_core_volume();
+      case kVolTensorEl: return tensor_core_volume_el();
       case kVolRegTab: return kVolRT;
       case kVolRegHalf: return kVolRH;
       default: return false;
@@ -235,6 +241,11 @@ class OpsImpl final : public Ops {
     if constexpr (kTcVol) {
       if (tc_ && (err = setup(k_volume_tc<D, K>, VolTc<D, K>::SMEM, VolTc<D, K>::THREADS, &g_vol_tc_, true)) !=
                      cudaSuccess)
+        return err;
+    }
+    if constexpr (kTcVolE) {
+      if (tc_ == 3 && (err = setup(k_volume_te<D, K>, VolTe<D, K>::SMEM, VolTe<D, K>::THREADS, &g_vol_te_, true)) !=
+                          cudaSuccess)
         return err;
     }
     if constexpr (kTcV2l) {
@@ -398,6 +409,15 @@ class OpsImpl final : public Ops {
   int volume(const DevMesh& m, const DevTabs& t, const void* uL, const void* wL, const void* gam,
              Combine c, void* out, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
+    if constexpr (kTcVolE) {
+      if (!wsep && vvar_ == kVolTensorEl && t.tcvole) {
+        using R = VolTe<D, K>;
+        launch(k_volume_te<D, K>, clamp_grid(g_vol_te_, m.E, R::TM), R::THREADS, R::SMEM, st, m,
+               static_cast<const unsigned char*>(t.tcvole), static_cast<const float*>(t.Wq), static_cast<const float*>(uL), static_cast<const float*>(gam),
+               static_cast<float*>(out), c);
+        return 1;
+      }
+    }
     if constexpr (kVolRH) {
       if (!wsep && (vvar_ == kVolRegHalf || !kVolR)) {
         using R = VolRH<D, K>;

@@ -76,6 +76,24 @@ __device__ __forceinline__ void mma_tf32_ts(uint32_t dtmem, uint32_t atmem, uint
       : "memory");
 }
 
+// Instruction descriptor of kind::f16 with BF16 operands: D in FP32 (bits 4-5 = 1), A and B
+// BF16 (bits 7-9, 10-12 = 1), both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// D[tmem] (+)= A[tmem] * B[smem]^T in BF16, issued by a single thread, K = 16: A is 128 TMEM lanes
+// x 8 columns of packed pairs (the lower index in the low half) from atmem; B core matrices are
+// 8 rows x 8 values.
+__device__ __forceinline__ void mma_f16_ts(uint32_t dtmem, uint32_t atmem, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dtmem),
+      "r"(atmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
 // Arrive once on the mbarrier when every MMA this thread issued before has completed.
 __device__ __forceinline__ void commit(uint64_t* mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -85,6 +103,10 @@ __device__ __forceinline__ void commit(uint64_t* mbar) {
 
 __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_test(uint64_t* mbar, uint32_t parity) {
@@ -152,6 +174,22 @@ __device__ __forceinline__ void ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 4 consecutive columns of four fields each, one wait for all (lane rule as ld16)
+__device__ __forceinline__ void ld4x4(const uint32_t (&taddr)[4], float (&v)[4][4]) {
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v[f][0]), "=f"(v[f][1]), "=f"(v[f][2]), "=f"(v[f][3])
+                 : "r"(taddr[f])
+                 : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0][0]), "+f"(v[0][1]), "+f"(v[0][2]), "+f"(v[0][3]), "+f"(v[1][0]), "+f"(v[1][1]),
+                 "+f"(v[1][2]), "+f"(v[1][3]), "+f"(v[2][0]), "+f"(v[2][1]), "+f"(v[2][2]), "+f"(v[2][3]),
+                 "+f"(v[3][0]), "+f"(v[3][1]), "+f"(v[3][2]), "+f"(v[3][3])
+               :
+               : "memory");
+}
+
 // ---------------------------------------------------------------- registers -> TMEM
 // N consecutive FP32 columns (N = 4, 8 or 16) of this thread's TMEM lane (same lane rule
 // as ld16); tmem_st_wait() makes them complete before a thread synchronisation hands the
@@ -196,6 +234,25 @@ __device__ __forceinline__ void tmem_st_cols(uint32_t taddr, const float* v) {
     if constexpr (W > 8) tmem_st_cols<W - 8>(taddr + 8, v + 8);
   } else {
     tmem_st<4>(taddr, v);
+  }
+}
+
+// N consecutive columns of raw registers, N even, in x8 / x4 / x2 pieces
+template <int N>
+__device__ __forceinline__ void tmem_st_u32(uint32_t taddr, const uint32_t* v) {
+  if constexpr (N >= 8) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+    if constexpr (N > 8) tmem_st_u32<N - 8>(taddr + 8, v + 8);
+  } else if constexpr (N >= 4) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
+                 "r"(v[2]), "r"(v[3])
+                 : "memory");
+    if constexpr (N > 4) tmem_st_u32<N - 4>(taddr + 4, v + 4);
+  } else {
+    static_assert(N == 2, "an even number of columns");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(taddr), "r"(v[0]), "r"(v[1]) : "memory");
   }
 }
 

@@ -256,6 +256,7 @@ class Hopu:
                        2: "warp per element, fused back-projection", 3: "tensor cores",
                        4: "register with gradient tables + separate back-projection",
                        5: "register, basis split over two lanes + separate back-projection",
+                       6: "tensor cores, elements along the rows + separate back-projection",
                        -1: "warp per element + separate back-projection"}
 
     def tuning_volume(self) -> dict:

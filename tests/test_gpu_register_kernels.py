@@ -12,7 +12,7 @@ import torch
 import workloads as W
 from oracle import adjoint as A
 from oracle import convection as C
-from oracle import fe, hdiv, mesh
+from oracle import fe, hdiv, mesh, rk
 
 pytestmark = pytest.mark.gpu
 
@@ -96,3 +96,48 @@ def test_vjp_per_facet_orders(dim, n, k):
     wb, ub = A.vjp_apply(topo, ref, sp.to_l2(wV), u, yb, fl.astype(np.int64))
     assert _rel(ubar, ub) < 2e-6
     assert _rel(wbar, sp.dual(wb)) < 2e-6
+
+
+@pytest.mark.parametrize("n,k,walls", [(3, 3, False), (4, 3, True), (5, 3, False), (3, 4, False), (4, 4, True), (5, 4, False)])
+def test_tensor_core_volume_rows(n, k, walls):
+    """The tensor-core volume kernel with elements along the rows (variant 6): element counts that
+    are no multiple of its tile of 40; the FP32 bounds of the operator (1e-6) and of a substep in
+    the parity tests (2e-6)."""
+    from paper_2408_06698_gb300 import Hopu
+    m = W.periodic_box_mesh(3, n)
+    rep = None if walls else m.rep
+    g = Hopu(m.coords, m.elems, rep, k=k, l=k - 1, prec="f32_tc")
+    topo, ref = mesh.MeshTopo(m.coords, m.elems, rep), fe.ref_element(3, k)
+    sp = hdiv.HDiv(topo, ref)
+    rng = np.random.default_rng(7900 + 10 * n + k)
+    u = sp.to_l2(rng.standard_normal(sp.n_hdiv)).astype(np.float32).astype(np.float64)
+    g.set_volume_variant(6)
+    assert g.tuning_volume()["variant"] == 6
+    ud = torch.as_tensor(u.reshape(-1), dtype=torch.float32, device=g.device)
+    y = g.apply_convection_l2(ud, ud)
+    g.sync()
+    assert _rel(y, C.apply(topo, ref, u, u, k - 1)) < 1e-6
+    v0 = rng.standard_normal(sp.n_hdiv).astype(np.float32).astype(np.float64)
+    a = torch.as_tensor(v0, dtype=torch.float32, device=g.device)
+    g.rk_substep(a, 1e-3, 1)
+    g.sync()
+    assert _rel(a, rk.substeps_stage(sp, v0, 1e-3, 1, k - 1)) < 2e-6
+    # a wait that gives up is reported, and the context recovers
+    g.set_wait_limit(0)
+    g.apply_convection_l2(ud, ud)
+    with pytest.raises(Exception, match="volume"):
+        g.sync()
+    g.clear_error()
+    g.set_wait_limit(None)
+    assert torch.equal(g.apply_convection_l2(ud, ud), y)
+    g.sync()
+
+
+def test_tensor_core_volume_rows_refused():
+    from paper_2408_06698_gb300 import Hopu
+    m = W.periodic_box_mesh(3, 3)
+    for k, prec in ((4, "f32"), (4, "tf32"), (2, "f32_tc"), (5, "f32_tc")):
+        g = Hopu(m.coords, m.elems, m.rep, k=k, l=k - 1, prec=prec)
+        with pytest.raises(Exception):
+            g.set_volume_variant(6)
+        g.close()
