@@ -94,9 +94,9 @@ typedef enum {
                         in twice the working precision), the geometry kept in FP64            */
   HOPU_FP32_TC = 2,  /* as HOPU_FP32, with dense contractions on the tensor cores in 3xTF32
                         (hi*hi + hi*lo + lo*hi, FP32 accumulation) where the autotuner finds
-                        them faster: the two dense products of the refined V_h -> L2
-                        projection (its residual stays compensated FP32 on the CUDA cores,
-                        so the projection keeps the accuracy of HOPU_FP32), the element part
+                        them faster: the V_h -> L2 projection (as products of base-256
+                        digits that are exact in BF16 and summed without rounding, so it
+                        keeps the accuracy of HOPU_FP32; 2D and 3D k <= 5), the element part
                         of the back-projection, and the STAGE volume contractions (3D k <= 3; 3D
                         k = 3, 4 also with three BF16 parts per operand and six products, an
                         error below FP32 rounding)
@@ -156,9 +156,8 @@ hopu_status hopu_destroy(hopu_ctx* ctx);
 hopu_status hopu_set_stream(hopu_ctx* ctx, void* cuda_stream);
 
 /* Kernel variants in use: out2[0] for the V_h -> L2 projection (HOPU_TF32: one TF32
- * product, k_v2l_tc; HOPU_FP32_TC: the refined projection with its two dense products on
- * the tensor cores and the compensated residual on the CUDA cores, k_v2l_tcr, 3D k <= 4
- * and 2D), out2[1] for the fused STAGE volume kernel; 0 = FP32 FMA kernel, 1 =
+ * product, k_v2l_tc, 3D k <= 4 and 2D; HOPU_FP32_TC: the product of exact digits,
+ * k_v2l_tcr), out2[1] for the fused STAGE volume kernel; 0 = FP32 FMA kernel, 1 =
  * tensor-core kernel.  No paper counterpart (launch tuning).                           */
 hopu_status hopu_tuning(const hopu_ctx* ctx, int* out2);
 

@@ -300,7 +300,7 @@ void free_all(hopu_ctx* c) {
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   void* ptrs[] = {c->d_elog_pos, c->d_mesh, c->d_geoT, c->d_geoF, c->d_tabs, c->d_gam, c->d_lf, c->d_uL, c->d_yL, c->d_wL,
                   c->d_wfz, c->d_s1, c->d_s2, c->d_diss, c->d_red, c->d_gamW, c->d_adj, c->d_err, c->d_tcvol, c->d_tcvole,
-                  c->d_inlet, c->d_inlet_modes, c->d_csr, c->d_tcl2v, c->d_tcv2l, c->d_csr_tc};
+                  c->d_inlet, c->d_inlet_modes, c->d_csr, c->d_tcl2v, c->d_tcv2l};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete c->ops;
@@ -422,7 +422,7 @@ void kernel_tables(const RefTables& R, bool fp64, std::vector<std::vector<double
 
 // The nonzeros of the dof matrix D (row s = functional, column r = basis function b*nb + i)
 // for the residual of the refined FP32 projection: nloc row headers {s, first entry, count,
-// grouped} (int32 bits) sorted by count, largest first, then one entry {r (int32 bits), hi, lo, 0}
+// 0} (int32 bits) sorted by count, largest first, then one entry {r (int32 bits), hi, lo, 0}
 // per nonzero with hi = float(D[s][r]), lo = float(D[s][r] - hi).  Entries below 1e-13 of
 // max |D| are the exact zeros of the orthogonality relations, rounded by the quadrature.
 std::vector<std::vector<std::pair<int, double>>> dof_matrix_rows(const RefTables& R) {
@@ -438,53 +438,12 @@ std::vector<std::vector<std::pair<int, double>>> dof_matrix_rows(const RefTables
   return rows;
 }
 
-// Rows whose dim component blocks are equal entry by entry (the facet whose reference
-// normal has equal components: D[s][b nb + i] = T[s][i] for every b) are grouped: only
-// block 0's nonzeros are kept (column i < nb) and D Y for the row is sum_i T[s][i] S_i with
-// S_i = sum_b Y[b nb + i].  Used by the refined tensor-core projection only.
-std::vector<bool> grouped_rows(const RefTables& R) {
-  const int nl = R.nloc, nb = R.nb, d = R.dim;
-  std::vector<bool> g(nl, false);
-  for (int s = 0; s < nl; ++s) {
-    bool eq = true;
-    for (int i = 0; i < nb && eq; ++i)
-      for (int b = 1; b < d; ++b)
-        if (R.D[(size_t)s * nl + b * nb + i] != R.D[(size_t)s * nl + i]) eq = false;
-    g[s] = eq;
-  }
-  return g;
-}
-
-// The order of the CSR rows: by number of stored nonzeros, largest first (stable).
-std::vector<int> csr_row_order(const RefTables& R, bool grouped) {
-  auto rows = dof_matrix_rows(R);
-  const std::vector<bool> g = grouped ? grouped_rows(R) : std::vector<bool>(R.nloc, false);
-  std::vector<size_t> cnt(R.nloc);
-  for (int s = 0; s < R.nloc; ++s) {
-    size_t c = 0;
-    for (const auto& e : rows[s]) c += (!g[s] || e.first < R.nb);
-    cnt[s] = c;
-  }
-  std::vector<int> order(R.nloc);
-  for (int s = 0; s < R.nloc; ++s) order[s] = s;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cnt[a] > cnt[b]; });
-  return order;
-}
-
-// grouped: rows with equal component blocks keep block 0 only and carry the flag 1 in the
-// fourth header word.
-void dof_matrix_csr(const RefTables& R, std::vector<float>& out, bool grouped = false) {
+void dof_matrix_csr(const RefTables& R, std::vector<float>& out) {
   const int nl = R.nloc;
-  auto rows = dof_matrix_rows(R);
-  const std::vector<int> order = csr_row_order(R, grouped);
-  const std::vector<bool> g = grouped ? grouped_rows(R) : std::vector<bool>(nl, false);
-  for (int s = 0; s < nl; ++s)
-    if (g[s]) {
-      std::vector<std::pair<int, double>> keep;
-      for (const auto& e : rows[s])
-        if (e.first < R.nb) keep.push_back(e);
-      rows[s] = keep;
-    }
+  const auto rows = dof_matrix_rows(R);
+  std::vector<int> order(nl);
+  for (int s = 0; s < nl; ++s) order[s] = s;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return rows[a].size() > rows[b].size(); });
   size_t nnz = 0;
   for (const auto& r : rows) nnz += r.size();
   out.assign(4 * (nl + nnz), 0.0f);
@@ -495,7 +454,6 @@ void dof_matrix_csr(const RefTables& R, std::vector<float>& out, bool grouped = 
     put_int(4 * h, s);
     put_int(4 * h + 1, next);
     put_int(4 * h + 2, (int)rows[s].size());
-    put_int(4 * h + 3, g[s] ? 1 : 0);
     for (const auto& e : rows[s]) {
       const float hi = (float)e.second;
       put_int(4 * (size_t)next, e.first);
@@ -608,25 +566,39 @@ void tensor_core_l2v_table(const RefTables& R, std::vector<float>& out) {
     }
 }
 
-// B operand of the refined tensor-core projection: B[r][kappa(h)] = Dinv[r][s_h] (r the basis
-// index, s_h the local functional of CSR row h, kappa(h) = (h % 4) GW + h / 4 the K column
-// of v2l_tc_gw), N = nloc padded to 16 rows; hi / lo TF32 parts, the hi parts then the lo
-// parts, blocked K-major as above.
-void tensor_core_v2l_table(const RefTables& R, std::vector<float>& out) {
-  const int nl = R.nloc, GW = v2l_tc_gw(nl), KP = v2l_tc_kp(nl), NP = (nl + 15) / 16 * 16;
-  const std::vector<int> order = csr_row_order(R, true);
-  const size_t P = (size_t)NP * KP;
-  out.assign(2 * P, 0.0f);
-  auto off = [&](int row, int col) {
-    return (size_t)(((row >> 3) * (KP >> 2) + (col >> 2)) * 32 + (row & 7) * 4 + (col & 3));
-  };
-  for (int r = 0; r < nl; ++r)
-    for (int h = 0; h < nl; ++h) {
-      const double v = R.Dinv[(size_t)r * nl + order[h]];
-      const float hi = tf32_round((float)v), lo = tf32_round((float)(v - (double)hi));
-      const int col = (h % 4) * GW + h / 4;
-      out[off(r, col)] = hi;
-      out[P + off(r, col)] = lo;
+// Table of the tensor-core projection: row n of Dinv divided by a power of two s_n (|values| < 128) as
+// base-256 digits d_0 + d_1 2^-8 + ..., |d| <= 128 in BF16, integers but for the last.  Per part of 16 GP columns (the
+// last may be narrower) digit j's rows follow digit j - 1's; column 16 g + d t + b is component b of
+// basis index g IPG + t; K is the local functional.  Core matrices of 8 rows x 8 values.  Then s_n / 256
+// of every column (FP32), zero where there is none.
+void tensor_core_v2l_table(const RefTables& R, std::vector<uint16_t>& out) {
+  const int nl = R.nloc, nb = R.nb, d = R.dim, KP = v2l_tc_kp(nl), IPG = v2l_tc_ipg(d), LV = kV2lLevels;
+  const int NGR = v2l_tc_groups(d, nb), GP = v2l_tc_part(d, nb, nl);
+  const size_t nB = (size_t)LV * 16 * NGR * KP;
+  out.assign(nB + (size_t)2 * 16 * NGR, 0);
+  for (int i = 0; i < nb; ++i)
+    for (int b = 0; b < d; ++b) {
+      const double* row = &R.Dinv[(size_t)(b * nb + i) * nl];
+      double mx = 0.0;
+      for (int s = 0; s < nl; ++s) mx = std::max(mx, std::fabs(row[s]));
+      int ex = 0;
+      std::frexp(mx, &ex);
+      const double scale = std::ldexp(1.0, ex - 7);
+      const int g = i / IPG, p = g / GP, nh = 16 * std::min(GP, NGR - p * GP);
+      const int c = 16 * (g - p * GP) + d * (i - g * IPG) + b;
+      for (int s = 0; s < nl; ++s) {
+        double v = row[s] / scale;
+        for (int j = 0; j < LV; ++j) {
+          const double q = j < LV - 1 ? std::nearbyint(v) : v;
+          const int r = j * nh + c;
+          double exact;
+          out[(size_t)p * LV * 16 * GP * KP + ((size_t)(r >> 3) * (KP >> 3) + (s >> 3)) * 64 + (r & 7) * 8 + (s & 7)] =
+              bf16_round(q, &exact);
+          v = (v - q) * 256.0;
+        }
+      }
+      const float f = (float)(scale / 256.0);
+      std::memcpy(&out[nB + 2 * (size_t)(16 * g + d * (i - g * IPG) + b)], &f, 4);
     }
 }
 
@@ -1024,16 +996,10 @@ hopu_status create_impl(const hopu_mesh_desc* mesh, const hopu_options* opts, vo
     c->dt.tcvole = c->d_tcvole;
   }
   if (c->ops->tensor_cores() && c->prec == HOPU_FP32_TC) {
-    std::vector<float> csr;
-    dof_matrix_csr(R, csr, true);
-    HOPU_CUDA(c, cudaMalloc(&c->d_csr_tc, csr.size() * sizeof(float)));
-    HOPU_CUDA(c, cudaMemcpy(c->d_csr_tc, csr.data(), csr.size() * sizeof(float), cudaMemcpyHostToDevice));
-    c->dt.Dcsr_tc = c->d_csr_tc;
-    c->dt.csr_tc_n = (int)(csr.size() / 4);
-    std::vector<float> tv;
+    std::vector<uint16_t> tv;
     tensor_core_v2l_table(R, tv);
-    HOPU_CUDA(c, cudaMalloc(&c->d_tcv2l, tv.size() * sizeof(float)));
-    HOPU_CUDA(c, cudaMemcpy(c->d_tcv2l, tv.data(), tv.size() * sizeof(float), cudaMemcpyHostToDevice));
+    HOPU_CUDA(c, cudaMalloc(&c->d_tcv2l, tv.size() * sizeof(uint16_t)));
+    HOPU_CUDA(c, cudaMemcpy(c->d_tcv2l, tv.data(), tv.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
     c->dt.tcv2l = c->d_tcv2l;
   }
   if (c->ops->tensor_core_l2v()) {

@@ -50,8 +50,6 @@ struct DevTabs {
   const void* Dcsr = nullptr;   // FP32: the nonzeros of D by rows, 16-byte entries (layout in
                                 //   k_v2l / warp_tile_residual); csr_n entries in all
   int csr_n = 0;
-  const void* Dcsr_tc = nullptr;  // FP32_TC: the same with grouped rows (rows whose component blocks are
-  int csr_tc_n = 0;               //   equal keep block 0 only, flag 1 in the header's fourth word)
   const void* DT = nullptr;     // [nloc][nlp]     DT[s][r]    = D[r][s]
   const void* Dinv = nullptr;   // [nloc][nlp]     Dinv[s][r]
   const void* Dn = nullptr;     // [nloc][nlp]     Dn[s][r] = D[s][r]
@@ -59,8 +57,8 @@ struct DevTabs {
                                 //   TF32 hi and lo parts), or NULL
   const void* Drow = nullptr;   // [nloc][nlr]     D[r][s] row-major, rows padded to nlr (an odd
                                 //                 multiple of 16 bytes), zero padding
-  const void* tcv2l = nullptr;  // FP32 3xTF32 refined projection table (Dinv as the B operand,
-                                //   TF32 hi and lo parts, layout of V2lTcr), or NULL
+  const void* tcv2l = nullptr;  // table of k_v2l_tcr (FP32_TC): Dinv's digits in BF16 as the B operands,
+                                //   then the scale of every column, or NULL
   const void* tcvole = nullptr; // tables of k_volume_te (FP32_TC, 3D k = 3, 4): the B operands in three
                                 //   BF16 parts each, or NULL
   const void* tcl2v = nullptr;  // FP32 tensor-core back-projection table (D as the B operand,
@@ -97,13 +95,17 @@ inline constexpr int l2v_tc_gw(int d, int nb) { return (d * l2v_tc_ipg(nb) + 3) 
 inline constexpr int l2v_tc_kp(int d, int nb) { return 4 * l2v_tc_gw(d, nb); }
 inline constexpr int l2v_tc_np(int nloc) { return (nloc + 15) / 16 * 16; }
 
-// K layout of the refined tensor-core projection (k_v2l_tcr and its host table): the rows h
-// of the sorted dof-matrix CSR (csr_row_order) are dealt to 4 warp groups, h = g + 4 j;
-// group g owns the RPG rows j and the K columns g GW + j (zero-padded to GW, a multiple
-// of 4); K = 4 GW; N = nloc padded to 16.
-inline constexpr int v2l_tc_rpg(int nloc) { return (nloc + 3) / 4; }
-inline constexpr int v2l_tc_gw(int nloc) { return (v2l_tc_rpg(nloc) + 3) / 4 * 4; }
-inline constexpr int v2l_tc_kp(int nloc) { return 4 * v2l_tc_gw(nloc); }
+// Sizes of the tensor-core projection (k_v2l_tcr and its host table): digits of the functionals,
+// digits of Dinv (= levels of the result); K padded to 16; the result's columns in groups of 16 (whole
+// basis indices, all components of each); groups of a part, whose levels fill TMEM beside the digits.
+inline constexpr int kV2lXDigits = 4, kV2lLevels = 5;
+inline constexpr int v2l_tc_kp(int nloc) { return (nloc + 15) / 16 * 16; }
+inline constexpr int v2l_tc_ipg(int d) { return 16 / d; }
+inline constexpr int v2l_tc_groups(int d, int nb) { return (nb + v2l_tc_ipg(d) - 1) / v2l_tc_ipg(d); }
+inline constexpr int v2l_tc_part(int d, int nb, int nloc) {
+  const int fit = (512 - kV2lXDigits * v2l_tc_kp(nloc) / 2) / (16 * kV2lLevels), g = v2l_tc_groups(d, nb);
+  return fit < 4 ? (fit < g ? fit : g) : (g < 4 ? g : 4);
+}
 
 // Sizes of the tensor-core volume kernel with elements along the rows (k_volume_te and its host
 // table): groups of warps, points per field padded to 4, K of the products padded to 16, columns of a

@@ -80,7 +80,6 @@ class OpsImpl final : public Ops {
   static constexpr bool kTcV2l = std::is_same<T, float>::value && V2lTc<D, K>::OK;
   static constexpr bool kTcV2lR = std::is_same<T, float>::value && V2lTcr<D, K>::OK;
   int g_v2l_tcr_ = 1;
-  bool tcr_fits_ = true;  // the CSR of D fits beside the refined tensor-core projection's tiles
   static constexpr bool kTcVol = std::is_same<T, float>::value && VolTc<D, K>::OK;
   int g_vol_tc_ = 1;
   // tensor-core STAGE volume kernel with elements along the rows (3xBF16 parts: HOPU_FP32_TC only)
@@ -194,10 +193,9 @@ class OpsImpl final : public Ops {
  public:
   explicit OpsImpl(int tc = 0) : tc_(std::is_same<T, float>::value ? tc : 0) { vvar_ = default_volume_variant(); }
   // The V_h -> L2 change of basis on the tensor cores: one TF32 product in TF32 mode
-  // (k_v2l_tc); in 3xTF32 mode the refined projection (k_v2l_tcr), whose two dense products
-  // run on the tensor cores and whose compensated residual keeps the small high-degree
-  // coefficients of smooth fields that a plain FP32 or 3xTF32 product loses.
-  bool tensor_cores() const override { return (tc_ == 1 && kTcV2l) || (tc_ == 3 && kTcV2lR && tcr_fits_); }
+  // (k_v2l_tc); in 3xTF32 mode the product of exact digits (k_v2l_tcr), which keeps the small
+  // high-degree coefficients of smooth fields that a plain FP32 or 3xTF32 product loses.
+  bool tensor_cores() const override { return (tc_ == 1 && kTcV2l) || (tc_ == 3 && kTcV2lR); }
   bool tensor_core_volume() const override { return tc_ != 0 && kTcVol; }
   bool tensor_core_volume_el() const override { return tc_ == 3 && kTcVolE; }
   void select(int v2l_tc, int volume_tc) override {
@@ -245,6 +243,11 @@ class OpsImpl final : public Ops {
     }
     if constexpr (kTcVolE) {
       if (tc_ == 3 && (err = setup(k_volume_te<D, K>, VolTe<D, K>::SMEM, VolTe<D, K>::THREADS, &g_vol_te_, true)) !=
+                          cudaSuccess)
+        return err;
+    }
+    if constexpr (kTcV2lR) {
+      if (tc_ == 3 && (err = setup(k_v2l_tcr<D, K>, V2lTcr<D, K>::SMEM, V2lTcr<D, K>::THREADS, &g_v2l_tcr_, true)) !=
                           cudaSuccess)
         return err;
     }
@@ -327,16 +330,6 @@ class OpsImpl final : public Ops {
   // The refined FP32 projection stages the sparse rows of D and, when they fit, Dinv^T per
   // CTA; as many warps per CTA as fit in ~220 KB (16, 12, 8 or 4).
   cudaError_t configure(const DevTabs& t) override {
-    if constexpr (kTcV2lR) {
-      if (tc_ == 3) {
-        const size_t sm = V2lTcr<D, K>::smem(t.csr_tc_n);
-        tcr_fits_ = sm <= 227 * 1024;
-        if (tcr_fits_) {
-          cudaError_t err = setup(k_v2l_tcr<D, K>, sm, V2lTcr<D, K>::THREADS, &g_v2l_tcr_, true);
-          if (err != cudaSuccess) return err;
-        }
-      }
-    }
     if constexpr (kRef) {
       using R = ProjRCfg<D, K>;
       csr_n_ = t.csr_n;
@@ -352,11 +345,10 @@ class OpsImpl final : public Ops {
 
   int v2l(const DevMesh& m, const DevTabs& t, const void* uV, void* uL, cudaStream_t st) override {
     if constexpr (kTcV2lR) {
-      if (tc_ == 3 && tcr_fits_ && use_tc_v2l_ && t.tcv2l && t.Dcsr_tc) {
+      if (tc_ == 3 && use_tc_v2l_ && t.tcv2l) {
         const int g = clamp_grid(g_v2l_tcr_, m.E, V2lTcr<D, K>::TM);
-        launch(k_v2l_tcr<D, K>, g, V2lTcr<D, K>::THREADS, V2lTcr<D, K>::smem(t.csr_tc_n), st, m,
-               static_cast<const float*>(t.tcv2l), static_cast<const float4*>(t.Dcsr_tc), t.csr_tc_n,
-               static_cast<const float*>(uV), static_cast<float*>(uL));
+        launch(k_v2l_tcr<D, K>, g, V2lTcr<D, K>::THREADS, V2lTcr<D, K>::SMEM, st, m,
+               static_cast<const unsigned char*>(t.tcv2l), static_cast<const float*>(uV), static_cast<float*>(uL));
         return 1;
       }
     }
