@@ -26,12 +26,14 @@
 // apart; what is dropped is 2^-24 of the product, below FP32 rounding, where 3xTF32 leaves 2^-21.
 //
 // Bound: the phases of a tile run one after another (one tile's D1 and A fill the TMEM at k = 4):
-// products 6.9 k, points 4.4 k, the rest 3.6 k of 14.9 k cycles.  12 worker warps (3 groups) of 128
+// products 5.2 k, points 4.4 k, the rest 3.6 k of 13.2 k cycles.  12 worker warps (3 groups) of 128
 // registers; 16 of them beside the MMA warp would leave 96 and spill.  A warp of its own issues the
 // MMAs: an issuing worker blocked 3 k cycles per tile on the tensor pipe's queue, and with it every
-// barrier.  Measured (CUDA events, per launch): 32^3 x 6, k = 4 528 us (k_volume_r) -> 239 us, on the
-// way 366 (one completion for all of D1, the lift on the CUDA cores, bound by its shared-memory
-// loads) and 330 (the lift as a product, halves); 16^3 x 6, k = 3 34 -> 28 us.  Error of the operator
+// barrier; its products are unrolled, with descriptors by increments (in a loop that built each
+// descriptor an MMA took its 80 cycles to issue).  Measured (CUDA events, per launch): 32^3 x 6, k = 4
+// 528 us (k_volume_r) -> 211 us, on the way 366 (one completion for all of D1, the lift on the CUDA
+// cores, bound by its shared-memory loads), 330 (the lift as a product, halves) and 239 (MMAs issued
+// from a loop); 16^3 x 6, k = 3 34 -> 26 us.  Error of the operator
 // against 64 bits, 32^3, k = 4: 3.6e-7 against 3.7e-7 with k_volume_r on Taylor-Green, 4.5e-7 against
 // 4.8e-7 on random coefficients.
 #pragma once
@@ -160,10 +162,10 @@ __global__ void __launch_bounds__(VolTe<D, K>::THREADS, K == 3 ? 2 : 1)
           const uint32_t b = sb1 + (h ? (4 * P0 / 8) * SB1 : 0);
 #pragma unroll
           for (int x = 0; x < 6; ++x)
-#pragma unroll 1
+#pragma unroll
             for (int ks = 0; ks < KP / 16; ++ks)
               tc::mma_f16_ts(tbase + (h ? 4 * P0 : 0), tbase + C::AO + PA[x] * (KP / 2) + 8 * ks,
-                             tc::sdesc(b + PB[x] * (uint32_t)C::B1 + 256 * ks, 128, SB1),
+                             tc::sdesc(b + PB[x] * (uint32_t)C::B1, 128, SB1) + 16 * ks,
                              tc::idesc_bf16(128, h ? 4 * P1 : 4 * P0), x > 0 || ks > 0);
           tc::commit(mb + 1 + h);
         }
@@ -177,13 +179,13 @@ __global__ void __launch_bounds__(VolTe<D, K>::THREADS, K == 3 ? 2 : 1)
 #pragma unroll
         for (int x = 0; x < 3; ++x) {
           const uint32_t id = tc::idesc_bf16(128, NN[x]);
-#pragma unroll 1
+#pragma unroll
           for (int ks = 0; ks < KG / 16; ++ks)
             tc::mma_f16_ts(tbase + C::DO + (x == 0 ? 1 : x) * NS, tbase + C::GO + x * GC + 8 * ks,
-                           tc::sdesc(sb3 + (x == 0 ? (NS / 8) * SB3 : 0) + 256 * ks, 128, SB3), id, x > 0 || ks > 0);
-#pragma unroll 1
+                           tc::sdesc(sb3 + (x == 0 ? (NS / 8) * SB3 : 0), 128, SB3) + 16 * ks, id, x > 0 || ks > 0);
+#pragma unroll
           for (int ks = 0; ks < KF / 16; ++ks)
-            tc::mma_f16_ts(tbase + C::DO + x * NS, tbase + x * FC + 8 * ks, tc::sdesc(sb2 + 256 * ks, 128, SB2), id, 1);
+            tc::mma_f16_ts(tbase + C::DO + x * NS, tbase + x * FC + 8 * ks, tc::sdesc(sb2, 128, SB2) + 16 * ks, id, 1);
         }
         tc::commit(mb + 3);
       }
