@@ -46,9 +46,9 @@ BOX16 = dict(dim=3, n=16, k=3, l=2, dt=5e-4, noise=1e-3, seed=0)
 # products on the tensor cores in 3xTF32 (the projection refined with a compensated FP32
 # residual), the facet and volume terms on the FP32 FMA kernels; autotuned per kernel family
 HEADLINE_PREC = "f32_tc"
-HEADLINE_MODE = ("HOPU_FP32_TC: FP32 data; 3xTF32 tensor-core products in the V_h -> L2 projection "
-                 "(refined by a compensated FP32 residual) and the back-projection, FP32 FMA facet and "
-                 "volume kernels; autotuned")
+HEADLINE_MODE = ("HOPU_FP32_TC: FP32 data; tensor-core V_h -> L2 projection (exact digit products), volume "
+                 "term (three BF16 parts, six products) and back-projection (3xTF32), FP32 FMA facet kernel; "
+                 "autotuned")
 APPLIES_PER_STEP = 3
 L2_FLUSH_BYTES = 256 << 20
 RESET_EVERY = 40  # substeps between restarts of the state from its initial value
