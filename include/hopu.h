@@ -326,6 +326,11 @@ hopu_status hopu_adapt_l(hopu_ctx* ctx, const void* u_l2, const double* threshol
  *   ubar_l2   = c(w; phi_j, z) for every L2 basis function phi_j (the transposed form);
  *   wbar_hdiv = E^T of d/dw c(w; u, z) tested with phi_j (E: V_h -> L2 of HOPU_HDIV_TO_L2),
  *               with d|s|/ds taken as 0 at s = w.n = 0.
+ * d|s|/ds jumps at s = 0.  At a facet point where |w.n| is below its rounding error (FP32: about
+ * one point in 10^7 for a wind that does not follow the mesh) the sign is that of w.n as summed
+ * in the working precision, in one fixed order (traces by basis index, then the normal's
+ * components, then the facet modes); wbar is then one of the two one-sided derivatives, and the
+ * other one is 1e-6 to 1e-4 of its norm away (16^3 x 6 tetrahedra).
  * Either output may be NULL (not both); outputs may not alias inputs or each other.
  * Layouts and working precision as hopu_apply_convection; asynchronous on the stream.  */
 hopu_status hopu_vjp_apply(hopu_ctx* ctx, const void* w_hdiv, const void* u_l2, const void* ybar_l2,

@@ -14,15 +14,45 @@
 // in registers; beta's low modes keep their normal part; alpha +- beta (sides A / B) go to the
 // ubar moments, gamma n_a to the wbar moments, scaled by a_F, element-major.
 //
+// sign(w.n) jumps at w.n = 0, and a point where |w.n| is no larger than its rounding error takes the
+// sign of that error: another order of the sums flips it, and one flipped point moves wbar by 1e-6 to
+// 1e-4 of its norm (16^3 x 6, k = 3: 4.1e-5 seen, two of a hundred random winds changed by more than
+// 2e-6).  So w.n has one order here and in k_facet_adj: a separate wind's traces by ascending basis
+// index, the normal component by ascending component, and, where the factorised value lies within the
+// rounding errors of the two ways to sum it, the sum over the modes themselves.  All lanes of a facet
+// then take one sign.  (w = u: the traces are those of u, in pairs.)
+//
 // Bound: FP32 FMA and shuffles.  Measured (CUDA events, per launch): separate wind 16^3 x 6 k = 3
-// 84 -> 44 us, 16^3 k = 4 261 -> 104 us, 10^3 k = 5 138 -> 49 us (a warp per facet before); w = u
+// 84 -> 44 us, 16^3 k = 4 261 -> 113 us, 10^3 k = 5 138 -> 54 us (a warp per facet before; 44, 100
+// and 49 us with the wind's traces in pairs, which other signs came with); w = u
 // 12^3 k = 3 27 -> 25 us (dense points, scalar FMAs and strided loads before), 10^3 k = 5 131 ->
-// 41 us.  At k = 5 about a hundred registers spill outside the point loop.
+// 41 us.  At k = 5 about twenty registers spill outside the point loop.
 #pragma once
 #include "kernels.cuh"
 #include "kernels_fr.cuh"
 
 namespace hopu {
+
+// A mode's trace as dot_ss sums it: every basis index, in order.  The entries of TrM that vanish by
+// degree are 1e-15 of quadrature rounding, and they count: 3 c, the trace of a degree 3 function's
+// coefficient alone, lies half-way between two FP32 values for every fourth c.
+template <int D, int K>
+__device__ __forceinline__ float facet_chain_trace(const float* row, const f2 (&c)[FacR<D, K>::NBP]) {
+  constexpr int NB = FacR<D, K>::NB;
+  float s = 0.0f;
+#pragma unroll
+  for (int i = 0; i < NB; i += 4) {
+    f2 t[2];
+    lds_f2(row + i, t[0], t[1]);
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      const int j = i + 2 * w;
+      if (j < NB) s = fmaf(f2_x(t[w]), f2_x(c[j / 2]), s);
+      if (j + 1 < NB) s = fmaf(f2_y(t[w]), f2_y(c[j / 2]), s);
+    }
+  }
+  return s;
+}
 
 template <int D, int K, bool WSEP>
 __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
@@ -51,6 +81,15 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
     if (D == 3) s += __shfl_sync(kFull, v, p2);
     return s;
   };
+  // v . n of a vector held by the facet's lanes, by ascending component: the same bits in every lane
+  auto normal = [&](float v, const float (&n)[D]) {
+    float s = 0.0f;
+#pragma unroll
+    for (int cc = 0; cc < D; ++cc) s = fmaf(__shfl_sync(kFull, v, fl * D + cc), n[cc], s);
+    return s;
+  };
+  auto half_sign = [](float v) { return (v > 0.0f) ? 0.5f : ((v < 0.0f) ? -0.5f : 0.0f); };
+  const float* Psi = static_cast<const float*>(tb.Psi);  // [NF][NQF], rule order q = i MF + j
   const int64_t ngroups = (m.NF + FPW - 1) / FPW, gstep = (int64_t)gridDim.x * C::WARPS;
   int64_t grp = (int64_t)warp * gridDim.x + blockIdx.x;
   int npa = 0, npb = 0;  // the next group's elements of this lane's facet
@@ -103,7 +142,7 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
       const float ju = tA - tB, av = 0.5f * (tA + tB);
       const float jn = lanes_sum(ju * na);
       UP[mm] = f2_pack(av, mm < nl ? jn * na : ju);
-      if (!WSEP) Wn[mm] = lanes_sum(av * na);
+      if (!WSEP) Wn[mm] = normal(av, n);
     }
     if (WSEP) next(wL, pa, pb, true);
     else next(uL, npa, npb, grp + gstep < ngroups);
@@ -118,11 +157,16 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
       next(uL, npa, npb, grp + gstep < ngroups);
 #pragma unroll
       for (int mm = 0; mm < NF; ++mm) {
-        const float tA = facet_plain_trace<D, K>(mm, trA + mm * NB4, cA, true);
-        const float tB = facet_plain_trace<D, K>(mm, trB + mm * NB4, cB, true);
-        Wn[mm] = lanes_sum((0.5f * (tA + tB)) * na);
+        const float tA = facet_chain_trace<D, K>(trA + mm * NB4, cA), tB = facet_chain_trace<D, K>(trB + mm * NB4, cB);
+        Wn[mm] = normal(0.5f * (tA + tB), n);
       }
     }
+    // the factorised w.n and the sum over the modes differ by at most (NF + 2 K + 6) roundings of
+    // sum_m |psi_m| |(w.n)_m|, and |psi_m| < 2 (K + 1) at the facet points
+    float near0 = 0.0f;
+#pragma unroll
+    for (int mm = 0; mm < NF; ++mm) near0 += fabsf(Wn[mm]);
+    near0 *= (NF + 2 * K + 6) * 2 * (K + 1) * 0x1p-24f;
     f2 ab[NF];
     float gs[NF];
 #pragma unroll
@@ -162,6 +206,7 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
           gw[p] = Wn[p];
         }
       }
+      float least = INFINITY;  // of |w.n| at the row's points
 #pragma unroll
       for (int i = 0; i < MF; ++i) {
         f2 A[K + 2], vu = f2_zero(), vz = f2_zero();
@@ -175,7 +220,8 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
           wn = fmaf(f2_x(A[p]), gw[p], wn);
         }
         const float hq = sWf[j * MF + i];         // w_q / 2
-        const float sg = (wn > 0.0f) ? 0.5f : ((wn < 0.0f) ? -0.5f : 0.0f);
+        least = fminf(least, fabsf(wn));
+        const float sg = half_sign(wn);
         const f2 pr = f2_mul(vu, vz);             // <u>_a [[z]]_a, (I - Pi)[[u]]_a (I - Pi)[[z]]_a
         const float s = hq * lanes_sum(fmaf(sg, f2_y(pr), f2_x(pr)));
         const float hw = hq * wn;
@@ -184,6 +230,31 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
         for (int p = 0; p <= K; ++p) {
           hs[p] = f2_fma(A[p], t, hs[p]);
           hg[p] = fmaf(f2_x(A[p]), s, hg[p]);
+        }
+      }
+      // a point whose sign the sum over the modes decides: about one in ten thousand, so the row is
+      // walked again for it (a branch per point parts the arithmetic of neighbouring points:
+      // 122 us for 113 at k = 4)
+      if (__any_sync(kFull, least <= near0)) {
+#pragma unroll 1
+        for (int i = 0; i < MF; ++i) {
+          f2 A[K + 2];
+          float wn = 0.0f, wm = 0.0f, vu = 0.0f, vz = 0.0f;
+#pragma unroll
+          for (int p = 0; p <= K; p += 2) lds_f2(sA + i * AST + 2 * p, A[p], A[p + 1]);
+#pragma unroll
+          for (int p = 0; p <= K; ++p) {
+            vu = fmaf(f2_x(A[p]), f2_y(gu[p]), vu);
+            vz = fmaf(f2_x(A[p]), f2_y(gz[p]), vz);
+            wn = fmaf(f2_x(A[p]), gw[p], wn);
+          }
+          const float* psi = Psi + (D == 3 ? i * MF + j : i);
+#pragma unroll
+          for (int mm = 0; mm < NF; ++mm) wm = fmaf(__ldg(psi + mm * C::NQF), Wn[mm], wm);
+          const float d = fabsf(wn) <= near0 ? half_sign(wm) - half_sign(wn) : 0.0f;
+          const float s = sWf[j * MF + i] * lanes_sum(d * (vu * vz));
+#pragma unroll
+          for (int p = 0; p <= K; ++p) hg[p] = fmaf(f2_x(A[p]), s, hg[p]);
         }
       }
       if constexpr (D == 3) {
