@@ -52,7 +52,9 @@ constexpr unsigned kFull = 0xffffffffu;
 // scheduled as soon as all of its own CTAs have started (pdl_trigger), and waits for the
 // previous kernel to complete, with its memory visible (pdl_wait), only after its
 // prologue, which reads nothing but constant tables and mesh data and writes only shared
-// memory.  Without the launch attribute both are no-ops.
+// memory.  Without the launch attribute both are no-ops.  A kernel that allocates TMEM triggers from
+// the allocating warp, after the allocation: a later kernel's CTA on the same SM could otherwise hold
+// the columns while it waits for this one, which would wait for the columns.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -55,7 +55,10 @@ __global__ void __launch_bounds__(256) k_v2l_tc(DevMesh m, const float* __restri
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double* geoT = m.geoT;
-  pdl_trigger();
+  if (warp == 0) {
+    tc::tmem_alloc(tslot, C::TCOLS);
+    pdl_trigger();  // behind the allocation, see pdl_trigger
+  }
 
   // B operand (once per CTA) and the zero padding columns of A
   for (int t = tid; t < NP * KP; t += NT) {
@@ -73,7 +76,6 @@ __global__ void __launch_bounds__(256) k_v2l_tc(DevMesh m, const float* __restri
       *reinterpret_cast<float*>(sAl + tc::blk_off(row, s, KP)) = 0.0f;
     }
   }
-  if (warp == 0) tc::tmem_alloc(tslot, C::TCOLS);
   if (tid == 0) {
     tc::mbar_init(mbar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -286,9 +288,10 @@ __global__ void __launch_bounds__(512, 1) k_volume_tc(DevMesh m, const float* __
   float* sCh = reinterpret_cast<float*>(sFl);                  // [EB][NL] (epilogue, F is free)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double* geoT = m.geoT;
-  pdl_trigger();
-
-  if (warp == 0) tc::tmem_alloc(tslot, C::TCOLS);
+  if (warp == 0) {
+    tc::tmem_alloc(tslot, C::TCOLS);
+    pdl_trigger();  // behind the allocation, see pdl_trigger
+  }
   if (tid == 0) {
     tc::mbar_init(mb_tab, 1);
     tc::mbar_init(mb_mma, 1);
@@ -573,9 +576,10 @@ __global__ void __launch_bounds__(512, 1) k_l2v_tc(DevMesh m, const float* __res
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = warp & 3, grp = warp >> 2;  // lane quarter, warp group
   const int el = q * 32 + lane;             // this thread's element (TMEM lane)
-  pdl_trigger();
-
-  if (warp == 0) tc::tmem_alloc(tslot, C::TCOLS);
+  if (warp == 0) {
+    tc::tmem_alloc(tslot, C::TCOLS);
+    pdl_trigger();  // behind the allocation, see pdl_trigger
+  }
   if (tid == 0) {
     tc::mbar_init(mb, 1);
     tc::mbar_init(mb + 1, 1);

@@ -103,9 +103,10 @@ __global__ void __launch_bounds__(V2lTcr<D, K>::THREADS, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = warp & 3, grp = warp >> 2;
   const int el = q * 32 + lane;  // this thread's element (TMEM lane)
-  pdl_trigger();
-
-  if (warp == 0) tc::tmem_alloc(tslot, C::TCOLS);
+  if (warp == 0) {
+    tc::tmem_alloc(tslot, C::TCOLS);
+    pdl_trigger();  // behind the allocation, see pdl_trigger
+  }
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < 5; ++i) tc::mbar_init(mb + i, 1);

@@ -127,8 +127,10 @@ __global__ void __launch_bounds__(VolTe<D, K>::THREADS, K == 3 ? 2 : 1)
   const int el = q4 * EPQ + le;                                     // the row's element of the tile
   const int a1 = (a + 1) % D, a2 = (a + 2) % D;
   const int p1 = lane_on ? le * D + a1 : lane, p2 = lane_on ? le * D + a2 : lane;
-  pdl_trigger();
-  if (warp == 0) tc::tmem_alloc(tslot, C::TCOLS);
+  if (warp == 0) {
+    tc::tmem_alloc(tslot, C::TCOLS);
+    pdl_trigger();  // behind the allocation, see pdl_trigger
+  }
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) tc::mbar_init(mb + i, 1);

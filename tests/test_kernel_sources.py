@@ -1,0 +1,39 @@
+"""Orders inside the CUDA kernels that no run can show to be kept: read from the sources.
+
+A kernel that allocates TMEM lets its successors start (programmatic dependent launch) only after
+the allocation.  The other way round a successor's CTA can take the columns of an SM first and then
+wait for the kernel whose CTA waits for those columns.
+"""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2408_06698_gb300", "csrc")
+
+
+def kernels(word):
+    """(file, text) of every __global__ function whose body holds `word`, comments removed."""
+    out = []
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith((".cuh", ".cu")):
+            text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+            out += [(name, part) for part in re.split(r"(?=__global__)", text)[1:] if word in part]
+    return out
+
+
+TMEM = kernels("tmem_alloc(")
+
+
+def test_tmem_kernels_are_found():
+    assert len(TMEM) >= 5
+
+
+@pytest.mark.parametrize("i", range(len(TMEM)))
+def test_dependents_start_after_the_tmem_allocation(i):
+    name, body = TMEM[i]
+    alloc, trigger = body.index("tmem_alloc("), body.index("pdl_trigger()")
+    assert trigger > alloc, name
+    # the same warp, in order: nothing but the end of the statement between the two
+    assert re.fullmatch(r"tmem_alloc\(tslot, C::TCOLS\);\s*pdl_trigger\(\)", body[alloc:trigger + len("pdl_trigger()")]), name
+    assert body.count("pdl_trigger()") == 1, name
