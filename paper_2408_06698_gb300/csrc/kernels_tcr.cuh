@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(V2lTcr<D, K>::THREADS, 1)
       const uint32_t sb = tc::smem_u32(smem_raw);
       const int64_t mine = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
       const uint32_t total = (uint32_t)(mine * PARTS);  // parts of this CTA; part c uses buffer c & 1
+      const uint32_t limit = tc::mma_warp_limit(m.tc_wait_limit);
       uint32_t c = 0, loaded = 0, ph = 0;
       auto load = [&] {
         if (!C::STREAM || loaded >= total) return;
@@ -142,15 +143,16 @@ __global__ void __launch_bounds__(V2lTcr<D, K>::THREADS, 1)
       load();
       load();
       bool go = true;
+      pdl_wait();
 #pragma unroll 1
       for (int64_t tile = blockIdx.x; go && tile < ntiles; tile += gridDim.x) {
 #pragma unroll 1
         for (int p = 0; p < PARTS; ++p, ph ^= 1u) {
-          go = tc::mbar_wait(mb + 2, ph, 1u << 24) && !*stop;
+          go = tc::mbar_wait(mb + 2, ph, limit) && !*stop;
           if (!go) break;
           if (C::STREAM) {
             if (c > 0) load();  // part c - 1 is done: the workers have read its result
-            go = tc::mbar_wait(mb + 3 + (c & 1), (c >> 1) & 1u, 1u << 24);
+            go = tc::mbar_wait(mb + 3 + (c & 1), (c >> 1) & 1u, limit);
             if (!go) break;
             ++c;
           }

@@ -153,10 +153,12 @@ __global__ void __launch_bounds__(VolTe<D, K>::THREADS, K == 3 ? 2 : 1)
   if (warp == NT / 32) {
     // the MMA warp: issuing blocks while the tensor pipe's queue is full, and no worker waits for it
     if (lane == 0 && ok) {
+      const uint32_t limit = tc::mma_warp_limit(m.tc_wait_limit);
       uint32_t ph = 0;
+      pdl_wait();
 #pragma unroll 1
       for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ph ^= 1u) {
-        if (!tc::mbar_wait(mb + 6, ph, 1u << 24) || *stop) break;
+        if (!tc::mbar_wait(mb + 6, ph, limit) || *stop) break;
         tc::fence_after_sync();
         constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};  // small products first
 #pragma unroll
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(VolTe<D, K>::THREADS, K == 3 ? 2 : 1)
                              tc::idesc_bf16(128, h ? 4 * P1 : 4 * P0), x > 0 || ks > 0);
           tc::commit(mb + 1 + h);
         }
-        if (!tc::mbar_wait(mb + 7, ph, 1u << 24) || *stop) break;
+        if (!tc::mbar_wait(mb + 7, ph, limit) || *stop) break;
         tc::fence_after_sync();
         // Part x of G and F against parts 0 .. 2 - x of B3 and B2, stacked along N, so that a block
         // of D2 takes the products of one order and no small product is rounded into a large sum.

@@ -129,6 +129,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint3
   return false;
 }
 
+// Polls of a warp that issues the MMAs and waits for the workers' operands, the workers' limit given:
+// at least 2^24 (about a second) and never fewer than theirs, so that the workers give up first and
+// report it.  The warp counts from the end of the previous kernel (pdl_wait), as the workers do: from
+// its own start the count would run while that kernel does.
+__device__ __forceinline__ uint32_t mma_warp_limit(uint32_t workers) { return workers > (1u << 24) ? workers : 1u << 24; }
+
 // ---------------------------------------------------------------- bulk copies (TMA, 1D)
 // Arm the mbarrier for `bytes` of incoming transactions (one arrival).
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {

@@ -3,6 +3,10 @@
 A kernel that allocates TMEM lets its successors start (programmatic dependent launch) only after
 the allocation.  The other way round a successor's CTA can take the columns of an SM first and then
 wait for the kernel whose CTA waits for those columns.
+
+A warp that only issues MMAs waits for the previous kernel before its first bounded wait for the
+workers, as the workers do, and follows the limit of hopu_set_wait_limit upwards: otherwise a long
+predecessor, or a raised limit, would make it give up work that was never late.
 """
 import os
 import re
@@ -37,3 +41,22 @@ def test_dependents_start_after_the_tmem_allocation(i):
     # the same warp, in order: nothing but the end of the statement between the two
     assert re.fullmatch(r"tmem_alloc\(tslot, C::TCOLS\);\s*pdl_trigger\(\)", body[alloc:trigger + len("pdl_trigger()")]), name
     assert body.count("pdl_trigger()") == 1, name
+
+
+MMA_WARP = kernels("warp == NT / 32")
+
+
+def test_mma_warp_kernels_are_found():
+    assert len(MMA_WARP) >= 2
+
+
+@pytest.mark.parametrize("i", range(len(MMA_WARP)))
+def test_mma_warp_waits(i):
+    name, body = MMA_WARP[i]
+    body = body[body.index("warp == NT / 32"):]
+    body = body[:body.index("} else {")]                # the MMA warp's branch
+    assert body.index("pdl_wait()") < body.index("mbar_wait("), name
+    assert "mma_warp_limit(m.tc_wait_limit)" in body, name
+    # the waits for the workers take that limit; only the final drain keeps the default
+    assert len(re.findall(r"mbar_wait\([^;]*, limit\)", body)) == 2, name
+    assert "1u << 24" not in body, name
