@@ -11,12 +11,13 @@ namespace hopu {
 struct DevMesh {
   int64_t E = 0, NF = 0;
   const double* geo = nullptr;   // [E][2d^2+2]: J (row-major), Jinv, det J, |det J| (FP64)
-  const double* geoT = nullptr;  // [E][geoT_stride(d)] FP64 in every precision mode (the FP32 kernels
-                                 // round each factor when they load it):
+  const double* geoT = nullptr;  // [E][geoT_stride(d)] FP64 in every precision mode:
                                  //   Pf = J / det J, Pi = det J * Jinv, M = |det J| * Jinv, 1/|det J|
-  const float* geoF = nullptr;   // FP32 contexts: geoT and fgeo rounded to FP32, same layouts.  A conversion
-  const float* fgeoF = nullptr;  // at the load runs on the FP64 unit: ten per thread were 3200 cycles of a
-                                 // 40-element tile of k_volume_te
+  const float* geoF = nullptr;   // FP32 contexts: geoT and fgeo rounded to FP32, same layouts, for the
+  const float* fgeoF = nullptr;  // register and tensor-core kernels (the warp-per-item kernels and the
+                                 // projections round a factor when they load it).  A conversion at the load
+                                 // runs on the FP64 unit: ten per thread were 3200 cycles of a 40-element
+                                 // tile of k_volume_te
   const int32_t* efc = nullptr;  // [E][d+1]: F*4 + (sigma<0)*2 + (element is side B)
   const int32_t* fa = nullptr;   // [NF]: element*4 + local facet of side A
   const int32_t* fb = nullptr;   // [NF]: same for side B

@@ -111,30 +111,34 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
     const int64_t eA = pa >> 2, eB = pb >> 2;
     const int fA = pa & 3, fB = pb & 3;
     sides(grp + gstep);
-    const double* fg = m.fgeo + F * (D + 1);
+    const float* fg = m.fgeoF + F * (D + 1);
     float n[D];
 #pragma unroll
-    for (int cc = 0; cc < D; ++cc) n[cc] = float(fg[cc]);
-    const float aF = float(fg[D]);
+    for (int cc = 0; cc < D; ++cc) n[cc] = __ldg(fg + cc);
+    const float aF = __ldg(fg + D);
     const float na = (a == 0) ? n[0] : (a == 1 ? n[1] : n[D - 1]);  // this lane's component of n
     const int l = facet_l ? int(facet_l[F]) : lconst;
     const int nl = (l < 0) ? 0 : cnbasis(D - 1, l);
-    const float iA = float(m.geoT[eA * GT + 3 * D * D]), iB = float(m.geoT[eB * GT + 3 * D * D]);
+    const float iA = __ldg(m.geoF + eA * GT + 3 * D * D), iB = __ldg(m.geoF + eB * GT + 3 * D * D);
     const float* trA = sTrM + fA * NF * NB4;
     const float* trB = sTrM + fB * NF * NB4;
     // both sides' coefficients of the field in the buffer; the next field's are requested
     f2 cA[NBP], cB[NBP];
-    auto next = [&](const float* src, int ra, int rb, bool more) {
-      cp_wait<0>();
-      __syncwarp();
-      facet_take<D, K>(sRec, 0, fl, a, eA, cA);
-      facet_take<D, K>(sRec, 1, fl, a, eB, cB);
-      __syncwarp();
-      if (more) facet_request<D, K>(src, sRec, ra, rb, lane);
+    auto next = [&](const float* cur, const float* src, int ra, int rb, bool more) {
+      if (C::STAGE) {
+        cp_wait<0>();
+        __syncwarp();
+      }
+      facet_take<D, K>(cur, sRec, 0, fl, a, eA, cA);
+      facet_take<D, K>(cur, sRec, 1, fl, a, eB, cB);
+      if (C::STAGE) {
+        __syncwarp();
+        if (more) facet_request<D, K>(src, sRec, ra, rb, lane);
+      }
     };
     f2 UP[NF], ZP[NF];  // (<u>, (I - Pi^l)[[u]]) and ([[z]], (I - Pi^l)[[z]]), modal
     float Wn[NF];
-    next(ybar, pa, pb, true);
+    next(uL, ybar, pa, pb, true);
 #pragma unroll
     for (int mm = 0; mm < NF; ++mm) {
       const float tA = facet_plain_trace<D, K>(mm, trA + mm * NB4, cA, true);
@@ -144,8 +148,8 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
       UP[mm] = f2_pack(av, mm < nl ? jn * na : ju);
       if (!WSEP) Wn[mm] = normal(av, n);
     }
-    if (WSEP) next(wL, pa, pb, true);
-    else next(uL, npa, npb, grp + gstep < ngroups);
+    if (WSEP) next(ybar, wL, pa, pb, true);
+    else next(ybar, uL, npa, npb, grp + gstep < ngroups);
 #pragma unroll
     for (int mm = 0; mm < NF; ++mm) {
       const float jz = iA * facet_plain_trace<D, K>(mm, trA + mm * NB4, cA, true) -
@@ -154,7 +158,7 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
       ZP[mm] = f2_pack(jz, mm < nl ? jn * na : jz);
     }
     if (WSEP) {
-      next(uL, npa, npb, grp + gstep < ngroups);
+      next(wL, uL, npa, npb, grp + gstep < ngroups);
 #pragma unroll
       for (int mm = 0; mm < NF; ++mm) {
         const float tA = facet_chain_trace<D, K>(trA + mm * NB4, cA), tB = facet_chain_trace<D, K>(trB + mm * NB4, cB);
@@ -235,7 +239,8 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
       // a point whose sign the sum over the modes decides: about one in ten thousand, so the row is
       // walked again for it (a branch per point parts the arithmetic of neighbouring points:
       // 122 us for 113 at k = 4)
-      if (__any_sync(kFull, least <= near0)) {
+      // (2D: the factorised sum is the sum over the modes)
+      if (D == 3 && __any_sync(kFull, least <= near0)) {
 #pragma unroll 1
         for (int i = 0; i < MF; ++i) {
           f2 A[K + 2];
@@ -248,7 +253,7 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, K <= 3 ? 3 : 2)
             vz = fmaf(f2_x(A[p]), f2_y(gz[p]), vz);
             wn = fmaf(f2_x(A[p]), gw[p], wn);
           }
-          const float* psi = Psi + (D == 3 ? i * MF + j : i);
+          const float* psi = Psi + i * MF + j;
 #pragma unroll
           for (int mm = 0; mm < NF; ++mm) wm = fmaf(__ldg(psi + mm * C::NQF), Wn[mm], wm);
           const float d = fabsf(wn) <= near0 ? half_sign(wm) - half_sign(wn) : 0.0f;

@@ -22,7 +22,7 @@
 // (alpha, beta) in the test, neighbouring basis indices in the traces.  A basis function of
 // degree n has a trace of degree <= n, so TrM[m][i] = 0 where deg psi_m > deg phi_i: those
 // products are left out, and only the modes of degree <= 1 have degree <= 1 terms to
-// compensate.  The coefficient records of a group's two sides arrive in shared memory by
+// compensate.  Where a record is long (STAGE) the records of a group's two sides arrive in shared memory by
 // 16-byte cp.async (one buffer per warp: the next group's records are requested as soon as
 // the current ones are in registers, and land during its points); loaded straight from
 // global memory, a lane's 35 consecutive values at k = 4 cost about 30 cache lines per
@@ -54,14 +54,19 @@ struct FacR {
   static constexpr int O_A = O_LOW + (D + 1) * (D + 1) * 4;      // [MF][AST]  A_p(t_i), each value twice
   static constexpr int O_B = O_A + MF * AST;                     // [MF][BST]  B_m(t_j), each value twice (3D)
   static constexpr int O_WF = O_B + MF * BST;                    // [NQF]      w_q / 2, i fastest
-  static constexpr int O_GEO = O_WF + r4i(NQF);                  // per warp: FPW (n, a_F), FP64
-  static constexpr int GEO = r4i(2 * FPW * (D + 1));
+  static constexpr int O_GEO = O_WF + r4i(NQF);                  // per warp: FPW (n, a_F)
+  static constexpr int GEO = r4i(FPW * (D + 1));
   static constexpr int O_REC = O_GEO + WARPS * GEO;              // per warp: 2 FPW coefficient records
   // a record starts at its element's offset modulo 16 bytes; strides keep scalar reads of
   // neighbouring lanes in different banks
   static constexpr int CH = (NL % 4 == 0 ? NL : r4i(NL + 3)) / 4;  // 16-byte chunks of a record
   static constexpr int RST = 4 * (CH % 2 ? CH : CH + 1);
-  static constexpr size_t SMEM = size_t(O_REC + WARPS * 2 * FPW * RST) * 4;
+  // 2D and k = 1: a lane's 3 to 15 coefficients of a side lie in one or two cache lines, and it loads
+  // them itself; through the buffer the SSP-RK3 substep of a 160^2 k = 1 square took 58.9 us (53.7), of
+  // 8^2 k = 4 43.9 (41.8), and a separate wind waited for its turn of the buffer (32 triangles, k = 4:
+  // 6.0 against 4.7 us an apply)
+  static constexpr bool STAGE = D == 3 && K > 1;
+  static constexpr size_t SMEM = size_t(O_REC + (STAGE ? WARPS * 2 * FPW * RST : 0)) * 4;
   static constexpr int REGS = 2 * NB + 3 * NF;                   // coefficients and the modal vectors
   static constexpr int MINB = REGS <= 120 ? 3 : 2;
 };
@@ -72,6 +77,10 @@ struct FacR {
 template <int D, int K>
 __device__ __forceinline__ void facet_request(const float* src, float* sRec, int pa, int pb, int lane) {
   using C = FacR<D, K>;
+  if (!C::STAGE) {
+    cp_commit();  // the geometry
+    return;
+  }
   constexpr int NL = C::NL, FPW = C::FPW, CH = C::CH, RST = C::RST;
   constexpr int RPI = CH <= 16 ? (CH <= 8 ? 4 : 2) : 1, LPR = 32 / RPI;
   const int cr = lane / LPR, cc0 = lane - cr * LPR;
@@ -97,12 +106,19 @@ __device__ __forceinline__ void facet_request(const float* src, float* sRec, int
   cp_commit();
 }
 
-// Component a of facet fl's record of one side, as pairs of neighbouring basis indices.
+// Component a of facet fl's record of one side, as pairs of neighbouring basis indices: from the
+// buffer, or (unless STAGE) from element e of src.
 template <int D, int K>
-__device__ __forceinline__ void facet_take(const float* sRec, int side, int fl, int a, int64_t e,
+__device__ __forceinline__ void facet_take(const float* src, const float* sRec, int side, int fl, int a, int64_t e,
                                            f2 (&c)[FacR<D, K>::NBP]) {
   using C = FacR<D, K>;
   constexpr int NB = C::NB, NL = C::NL;
+  if constexpr (!C::STAGE) {
+    const float* p = src + e * NL + a * NB;
+#pragma unroll
+    for (int j = 0; j < C::NBP; ++j) c[j] = f2_pack(__ldg(p + 2 * j), 2 * j + 1 < NB ? __ldg(p + 2 * j + 1) : 0.0f);
+    return;
+  }
   const float* p = sRec + (side * C::FPW + fl) * C::RST + a * NB;
   if constexpr (NL % 4 == 0 && NB % 4 == 0) {
 #pragma unroll
@@ -189,7 +205,7 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
   const float* sWf = sm + C::O_WF;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* sRec = sm + C::O_REC + warp * 2 * FPW * RST;
-  const double* sGeo = reinterpret_cast<const double*>(sm + C::O_GEO + warp * C::GEO);
+  float* sGeo = sm + C::O_GEO + warp * C::GEO;
   const bool lane_on = lane < D * FPW;
   const int fl = lane_on ? lane / D : 0;
   const int a = lane_on ? lane - fl * D : 0;
@@ -202,7 +218,7 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
   };
   const int64_t ngroups = (m.NF + FPW - 1) / FPW, gstep = (int64_t)gridDim.x * C::WARPS;
   auto request = [&](const float* src, int pa, int pb) { facet_request<D, K>(src, sRec, pa, pb, lane); };
-  auto take = [&](int side, int64_t e, f2 (&c)[NBP]) { facet_take<D, K>(sRec, side, fl, a, e, c); };
+  auto take = [&](const float* src, int side, int64_t e, f2 (&c)[NBP]) { facet_take<D, K>(src, sRec, side, fl, a, e, c); };
   auto plain = [&](int mm, const float* row, const f2 (&c)[NBP], bool all) {
     return facet_plain_trace<D, K>(mm, row, c, all);
   };
@@ -218,7 +234,7 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
   auto request_geo = [&](int64_t g) {
     const int64_t i0 = g * FPW * (D + 1), end = m.NF * (D + 1);
     for (int t = lane; t < FPW * (D + 1); t += 32)
-      if (i0 + t < end) cp_async<8>(const_cast<double*>(sGeo) + t, m.fgeo + i0 + t);
+      if (i0 + t < end) cp_async<4>(sGeo + t, m.fgeoF + i0 + t);
   };
   sides(grp);
   if (grp < ngroups) request_geo(grp);  // mesh data: before the wait for the previous kernel
@@ -246,13 +262,13 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
       f2 cA[NBP], cB[NBP];
       cp_wait<0>();
       __syncwarp();
-      take(0, eA, cA);
-      take(1, eB, cB);
+      take(uL, 0, eA, cA);
+      take(uL, 1, eB, cB);
       {
-        const double* fg = sGeo + (act ? fl : 0) * (D + 1);
+        const float* fg = sGeo + (act ? fl : 0) * (D + 1);
 #pragma unroll
-        for (int cc = 0; cc < D; ++cc) n[cc] = float(fg[cc]);
-        aF = float(fg[D]);
+        for (int cc = 0; cc < D; ++cc) n[cc] = fg[cc];
+        aF = fg[D];
         na = (a == 0) ? n[0] : (a == 1 ? n[1] : n[D - 1]);
       }
       __syncwarp();
@@ -309,11 +325,13 @@ __global__ void __launch_bounds__(32 * FacR<D, K>::WARPS, FacR<D, K>::MINB)
     }
     if (WSEP) {  // the wind's traces from its own coefficients
       f2 wA[NBP], wB[NBP];
-      cp_wait<0>();
-      __syncwarp();
-      take(0, eA, wA);
-      take(1, eB, wB);
-      __syncwarp();
+      if (C::STAGE) {
+        cp_wait<0>();
+        __syncwarp();
+      }
+      take(wL, 0, eA, wA);
+      take(wL, 1, eB, wB);
+      if (C::STAGE) __syncwarp();
       if (grp + gstep < ngroups) request(uL, npa, npb);
 #pragma unroll
       for (int mm = 0; mm < NF; ++mm) {

@@ -124,19 +124,19 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, MODE>::WARPS, VolRH<D, K, MOD
     const int ne = count(grp);
     const bool act = lane_on && el < ne;
     const int64_t e = act ? e0 + el : e0;  // inactive lanes read the group's first element
-    const double* gp = m.geoT + e * GT;
+    const float* gp = m.geoF + e * GT;
     // M = |det J| J^-1: its columns a, a + 1, a + 2 (w = u), column a (kVolAdjW) or row a in M0
     constexpr bool COLS = MODE == kVolSame || MODE == kVolAdjSame;
     float M0[D], M1[COLS ? D : 1], M2[COLS ? D : 1];
 #pragma unroll
     for (int cc = 0; cc < D; ++cc) {
-      M0[cc] = float(__ldg(gp + 2 * D * D + (ROW ? a * D + cc : cc * D + a)));
+      M0[cc] = __ldg(gp + 2 * D * D + (ROW ? a * D + cc : cc * D + a));
       if constexpr (COLS) {
-        M1[cc] = float(__ldg(gp + 2 * D * D + cc * D + a1));
-        M2[cc] = D == 3 ? float(__ldg(gp + 2 * D * D + cc * D + a2)) : 0.0f;
+        M1[cc] = __ldg(gp + 2 * D * D + cc * D + a1);
+        M2[cc] = D == 3 ? __ldg(gp + 2 * D * D + cc * D + a2) : 0.0f;
       }
     }
-    const float invabs = float(__ldg(gp + 3 * D * D));
+    const float invabs = __ldg(gp + 3 * D * D);
     // this half's coefficients, entries 2 t + h (zero beyond the half): c those whose gradient is
     // taken, ev those evaluated at the points (as in k_volume_r)
     f2 c[NP], ev[MODE == kVolSame ? 1 : NP];

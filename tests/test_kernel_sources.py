@@ -60,3 +60,24 @@ def test_mma_warp_waits(i):
     # the waits for the workers take that limit; only the final drain keeps the default
     assert len(re.findall(r"mbar_wait\([^;]*, limit\)", body)) == 2, name
     assert "1u << 24" not in body, name
+
+
+def members(struct):
+    """Names of the data members of a struct of hopu_internal.h."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "hopu_internal.h")).read())
+    body = text[text.index(f"struct {struct} {{"):]
+    body = body[:body.index("};")]
+    return re.findall(r"\b(\w+)\s*=", body)
+
+
+@pytest.mark.parametrize("struct,var", [("DevMesh", "m")])
+def test_every_array_of_a_context_is_read(struct, var):
+    """What a context uploads and passes to every launch is read by a kernel or named at a launch."""
+    text = "".join(re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, n)).read()) for n in sorted(os.listdir(CSRC))
+                   if n.endswith(".cuh"))
+    capi = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "capi.cu")).read())
+    names = members(struct)
+    assert len(names) >= 8
+    for name in names:
+        read = re.search(rf"\b(?:{var}|t)\.{name}\b", text) or re.search(rf"c->dm\.{name}\b(?!\s*=[^=])", capi)
+        assert read, f"{struct}::{name}"
