@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_facet_adj(DevMesh m, DevTabs tb
 }
 
 // Volume part of the adjoint plus the lift of the facet moments.  WSEP: separate wind
-// (outputs ubar and wbar); otherwise w = u and the two cotangents are summed into ubar.
+// (outputs ubar and wbar, either may be NULL); otherwise w = u and the two cotangents are summed into ubar.
 template <int D, int K, typename T, bool WSEP>
 __global__ void __launch_bounds__(32 * kWarps) k_volume_adj(DevMesh m, DevTabs tb, const T* __restrict__ uL,
                                                             const T* __restrict__ wL, const T* __restrict__ ybar,
@@ -327,8 +327,8 @@ __global__ void __launch_bounds__(32 * kWarps) k_volume_adj(DevMesh m, DevTabs t
           rw = fma(t, sGW[fm * D + a], rw);
         }
         if constexpr (WSEP) {
-          ubar[e * NL + idx] = ru;
-          wbar[e * NL + idx] = accW[j] + rw;
+          if (ubar) ubar[e * NL + idx] = ru;
+          if (wbar) wbar[e * NL + idx] = accW[j] + rw;
         } else {
           ubar[e * NL + idx] = ru + rw;
         }

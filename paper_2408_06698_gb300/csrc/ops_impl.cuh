@@ -130,9 +130,27 @@ class OpsImpl final : public Ops {
              static_cast<const float*>(ybar), static_cast<const float*>(gam), static_cast<const float*>(gam2),
              static_cast<float*>(out), Combine());
   }
+  // Separate wind on a small mesh (FP32): a warp per facet or element.  A register warp walks the points of
+  // its 10 to 16 items one after another, which takes longer than the one pass of a warp per item; the
+  // limits are items per SM.  us per call (graph of 20 calls), warp per item / register kernel:
+  //   facet term, apply: 3D k = 4, 324 facets 17.1 / 22.1, 1500 27.3 / 28.1, 2592 33.0 / 31.8; k = 5, 324
+  //     40.5 / 48.1, 768 (two CTAs on some SMs, each with its own tables) 53.0 / 44.1; 2D k = 3, 768
+  //     4.3 / 5.0, 1728 6.7 / 5.6; k = 4, 768 5.8 / 5.9, 1728 7.5 / 7.1; other orders at most even;
+  //   facet part of the VJP: 3D k = 2, 324 20.3 / 22.1, 1500 24.4 / 25.4, 6144 31.0 / 29.7; 2D k = 4, 48
+  //     17.6 / 18.4, 1728 20.0 / 19.8; other orders at most 2 % apart at the smallest mesh;
+  //   volume part of the VJP: 2D k = 4, 32 elements 18.4 / 26.9, 4608 29.5 / 31.6, 8192 37.4 / 34.5; k = 3, 4608
+  //     20.2 / 22.3; k = 2, 512 11.9 / 14.1, 1152 13.1 / 14.2; 3D k = 2, 162 22.1 / 27.9, 4374 30.8 / 33.2, 6000
+  //     35.7 / 35.2; k = 1, 384 13.7 / 14.7, 750 14.7 / 14.9; from 3D k = 3 on its sums spill (162 elements, 80 /
+  //     45).  One cotangent alone takes the same kernel (the same bits) although the register kernel then runs
+  //     once (2D k = 2, 2048 11.7 / 8.5): the lines of k = 1 and of 2D k = 2 lie lower for it.
+  static constexpr int kFacSmall = D == 3 ? (K == 4 ? 12 : K == 5 ? 4 : 0) : (K >= 3 ? 8 : 0);
+  static constexpr int kFacAdjSmall = (D == 3 && K == 2) || (D == 2 && K == 4) ? 10 : 0;
+  static constexpr int kVolAdjSmall = K == 1 ? 4 : D == 2 ? (K == 2 ? 8 : 32) : K == 2 ? 32 : 0;
+  bool small(int64_t items, int per_sm) const { return items <= (int64_t)per_sm * nsm_; }
   int g_facar_[2] = {1, 1};  // facet part of the VJP in FP32: w = u, separate wind
   int g_volr_ = 1, g_volrf_ = 1;
-  // facet term: register-resident kernel in FP32 (every order), a warp per facet in FP64
+  // facet term: register-resident kernel in FP32 (every order), a warp per facet in FP64 and on small
+  // meshes
   static constexpr bool kFacR = std::is_same<T, float>::value;
   int g_facr_[2] = {1, 1};
   int g_v2l_ = 1, g_v2lpt_ = 1, g_fac_[2] = {1, 1}, g_vol_[2] = {1, 1}, g_elem_[2] = {1, 1}, g_fsum_ = 1;
@@ -273,6 +291,12 @@ class OpsImpl final : public Ops {
       if ((err = setup_adj<kVolAdjU>()) != cudaSuccess) return err;
       if ((err = setup_adj<kVolAdjW>()) != cudaSuccess) return err;
       if ((err = setup_adj<kVolAdjSame>()) != cudaSuccess) return err;
+      if constexpr (kFacAdjSmall) {
+        if ((err = setup(k_facet_adj<D, K, T, true>, facet_adj_smem(true), th, &g_fadj_)) != cudaSuccess) return err;
+      }
+      if constexpr (kVolAdjSmall) {
+        if ((err = setup(k_volume_adj<D, K, T, true>, volume_adj_smem(true), th, &g_vadj_)) != cudaSuccess) return err;
+      }
     } else {
       if ((err = setup(k_facet_adj<D, K, T, false>, facet_adj_smem(false), th, &g_fadj_)) != cudaSuccess) return err;
       if ((err = setup(k_facet_adj<D, K, T, true>, facet_adj_smem(true), th, &g_fadj_)) != cudaSuccess) return err;
@@ -286,6 +310,8 @@ class OpsImpl final : public Ops {
     }
     if constexpr (!kFacR) {
       if ((err = setup(k_facet<D, K, T, false, kFacetTab>, facet_smem(false), th, &g_fac_[0])) != cudaSuccess) return err;
+    }
+    if constexpr (!kFacR || kFacSmall) {
       if ((err = setup(k_facet<D, K, T, true, kFacetTab>, facet_smem(true), th, &g_fac_[1])) != cudaSuccess) return err;
     }
     if constexpr (!std::is_same<T, float>::value) {
@@ -378,6 +404,13 @@ class OpsImpl final : public Ops {
             const int8_t* facet_l, void* gam, double* diss, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (kFacR) {
+      if constexpr (kFacSmall) {
+        if (wsep && small(m.NF, kFacSmall)) {
+          launch(k_facet<D, K, T, true, kFacetTab>, clamp_grid(g_fac_[1], m.NF, kWarps), 32 * kWarps, facet_smem(true), st,
+              m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), l, facet_l, static_cast<T*>(gam), diss);
+          return 1;
+        }
+      }
       using R = FacR<D, K>;
       const int g = clamp_grid(g_facr_[wsep ? 1 : 0], (m.NF + R::FPW - 1) / R::FPW, 1);
       if (wsep)
@@ -495,6 +528,14 @@ class OpsImpl final : public Ops {
                 const int8_t* facet_l, void* gamU, void* gamW, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (std::is_same<T, float>::value) {
+      if constexpr (kFacAdjSmall) {
+        if (wsep && small(m.NF, kFacAdjSmall)) {
+          launch(k_facet_adj<D, K, T, true>, clamp_grid(g_fadj_, m.NF, kWarps), 32 * kWarps, facet_adj_smem(true), st,
+              m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar), l, facet_l,
+              static_cast<T*>(gamU), static_cast<T*>(gamW));
+          return 1;
+        }
+      }
       using R = FacR<D, K>;
       const int g = clamp_grid(g_facar_[wsep ? 1 : 0], (m.NF + R::FPW - 1) / R::FPW, 1);
       if (wsep)
@@ -526,6 +567,14 @@ class OpsImpl final : public Ops {
       if (!wsep) {
         launch_adj<kVolAdjSame>(m, t, uL, ybar, gamU, gamW, ubar, st);
         return 1;
+      }
+      if constexpr (kVolAdjSmall) {
+        if (small(m.E, kVolAdjSmall)) {
+          launch(k_volume_adj<D, K, T, true>, clamp_grid(g_vadj_, m.E, kWarps), 32 * kWarps, volume_adj_smem(true), st,
+              m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar),
+              static_cast<const T*>(gamU), static_cast<const T*>(gamW), static_cast<T*>(ubar), static_cast<T*>(wbar));
+          return 1;
+        }
       }
       if (ubar) launch_adj<kVolAdjU>(m, t, wL, ybar, gamU, nullptr, ubar, st);
       if (wbar) launch_adj<kVolAdjW>(m, t, uL, ybar, gamW, nullptr, wbar, st);
