@@ -315,7 +315,7 @@ void convert(const std::vector<double>& src, std::vector<unsigned char>& dst, si
 }
 
 // Reorder the host FP64 tables into the kernel layouts (see hopu_internal.h).
-constexpr int kNumTables = 16;
+constexpr int kNumTables = 15;
 
 // Row stride of the point-major tables: an odd multiple of 16 bytes (matches
 // row_stride<T> in kernels.cuh).
@@ -333,7 +333,7 @@ void kernel_tables(const RefTables& R, bool fp64, std::vector<std::vector<double
   auto& Wq = out[1];
   auto& Dm = out[2];
   auto& TrM = out[3];
-  auto& TrP = out[4];
+  auto& FacB = out[4];
   auto& Psi = out[5];
   auto& WPsi = out[6];
   auto& Wf = out[7];
@@ -367,10 +367,6 @@ void kernel_tables(const RefTables& R, bool fp64, std::vector<std::vector<double
         dBt[((size_t)c * nqk + q) * nbq + i] = acc;
       }
   TrM = R.trm;
-  TrP.assign((size_t)(d + 1) * nqf * nbq, 0.0);  // point-major [f][q][nbq]
-  for (int f = 0; f <= d; ++f)
-    for (int q = 0; q < nqf; ++q)
-      for (int i = 0; i < nb; ++i) TrP[((size_t)f * nqf + q) * nbq + i] = R.phif[((size_t)f * nqf + q) * nb + i];
   Psi.resize((size_t)nf * nqf);
   WPsi.resize((size_t)nf * nqf);
   for (int m = 0; m < nf; ++m)
@@ -383,7 +379,6 @@ void kernel_tables(const RefTables& R, bool fp64, std::vector<std::vector<double
   // orthonormal Legendre polynomial of the first direction, B_m = psi_m / A_p taken where
   // |A_p| is largest (a constant along the first direction)
   auto& FacA = out[14];
-  auto& FacB = out[15];
   const int mf = rule_m(3 * R.k), K1 = R.k + 1;
   std::vector<double> t1, w1;
   gauss_jacobi01(mf, 0, t1, w1);
@@ -969,9 +964,9 @@ hopu_status create_impl(const hopu_mesh_desc* mesh, const hopu_options* opts, vo
   HOPU_CUDA(c, cudaMemcpy(c->d_tabs, ht.data(), total, cudaMemcpyHostToDevice));
   unsigned char* tb = static_cast<unsigned char*>(c->d_tabs);
   const void** slots[kNumTables] = {&c->dt.Bt,   &c->dt.Wq,  &c->dt.Dm,    &c->dt.TrM,
-                                    &c->dt.TrP,  &c->dt.Psi, &c->dt.WPsi,  &c->dt.Wf,
+                                    &c->dt.FacB,  &c->dt.Psi, &c->dt.WPsi,  &c->dt.Wf,
                                     &c->dt.DinvT, &c->dt.DT, &c->dt.Dinv, &c->dt.Drow, &c->dt.Dn,
-                                    &c->dt.dBt, &c->dt.FacA, &c->dt.FacB};
+                                    &c->dt.dBt, &c->dt.FacA};
   for (int i = 0; i < kNumTables; ++i) *slots[i] = tb + offs[i];
   if (!c->fp64) {
     std::vector<float> csr;

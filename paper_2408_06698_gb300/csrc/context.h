@@ -15,7 +15,7 @@ struct hopu_ctx {
   using MeshTopo = hopu::MeshTopo;
   using RefTables = hopu::RefTables;
   using DevMesh = hopu::DevMesh;
-  using DevTabs = hopu::DevTabs;
+  using LaunchTabs = hopu::LaunchTabs;
   using Ops = hopu::Ops;
   int dim = 0, k = 0, l = -1, prec = 0, wind = 0;
   bool fp64 = true;
@@ -25,7 +25,7 @@ struct hopu_ctx {
   RefTables ref;
   int64_t n_hdiv = 0, n_l2 = 0;
   DevMesh dm;
-  DevTabs dt;
+  LaunchTabs dt;
   Ops* ops = nullptr;
   int nsm = 1, red_blocks = 1;
   double l2v_ms[2] = {-1.0, -1.0};  // autotuner: ms per launch of the FMA / tensor-core back-projection

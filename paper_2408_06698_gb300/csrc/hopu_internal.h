@@ -32,7 +32,9 @@ struct DevMesh {
   const void* inlet_modes = nullptr;  // [n_inlet][nf][d] modal exterior trace, working precision
 };
 
-// Device reference tables in working precision (all element-type T, 16-byte aligned).
+// Device reference tables in working precision (all element-type T, 16-byte aligned) that kernels take
+// as one argument.  Every launch copies its arguments: 40 bytes more cost the 150 launches of ten
+// substeps of an 8 x 8 square 0.8 % (706 -> 711 us), so a table that only a launch names is in LaunchTabs.
 struct DevTabs {
   const void* Bt = nullptr;     // [nq][nbq]       phi_i(x_q), point-major, rows padded to nbq
   const void* dBt = nullptr;    // [d][nq][nbq]    d phi_i / d xhat_c (x_q), same layout as Bt
@@ -40,13 +42,18 @@ struct DevTabs {
   const void* Wq = nullptr;     // [nq]            volume weights
   const void* Dm = nullptr;     // [d][nb(k-1)][nb] d phi_i / d xhat_c = sum_j Dm[c][j][i] phi_j
   const void* TrM = nullptr;    // [d+1][nf][nb]   <phi_i o xhat_f, psi_m>_facet
-  const void* TrP = nullptr;    // [d+1][nqf][nbq] phi_i(xhat_f(s_q)), point-major
   const void* Psi = nullptr;    // [nf][nqf]       psi_m(s_q)
   const void* WPsi = nullptr;   // [nf][nqf]       w_q psi_m(s_q)
   const void* Wf = nullptr;     // [nqf]           facet weights
   const void* FacA = nullptr;   // [mf][k+1]       facet basis factors at the points (t_i, t_j) of the facet
   const void* FacB = nullptr;   // [mf][nf]          rule: psi_m = A_p(t_i) B_m(t_j), p the first index of
                                 //                 mode m (2D: psi_p = A_p, B = 1)
+  const void* Drow = nullptr;   // [nloc][nlr]     D[r][s] row-major, rows padded to nlr (an odd
+                                //                 multiple of 16 bytes), zero padding
+};
+
+// The tables and what a launch passes by itself.
+struct LaunchTabs : DevTabs {
   const void* DinvT = nullptr;  // [nloc][nlp]     DinvT[s][r] = Dinv[r][s]  (nlp = nloc rounded up to 4)
   const void* Dcsr = nullptr;   // FP32: the nonzeros of D by rows, 16-byte entries (layout in
                                 //   k_v2l / warp_tile_residual); csr_n entries in all
@@ -56,8 +63,6 @@ struct DevTabs {
   const void* Dn = nullptr;     // [nloc][nlp]     Dn[s][r] = D[s][r]
   const void* tcvol = nullptr;  // FP32 tensor-core volume tables (phi in the two operand layouts,
                                 //   TF32 hi and lo parts), or NULL
-  const void* Drow = nullptr;   // [nloc][nlr]     D[r][s] row-major, rows padded to nlr (an odd
-                                //                 multiple of 16 bytes), zero padding
   const void* tcv2l = nullptr;  // table of k_v2l_tcr (FP32_TC): Dinv's digits in BF16 as the B operands,
                                 //   then the scale of every column, or NULL
   const void* tcvole = nullptr; // tables of k_volume_te (FP32_TC, 3D k = 3, 4): the B operands in three
@@ -147,22 +152,22 @@ class Ops {
   virtual ~Ops() {}
   virtual cudaError_t prepare() = 0;
   // launch configuration that depends on the uploaded tables (after prepare)
-  virtual cudaError_t configure(const DevTabs&) = 0;
+  virtual cudaError_t configure(const LaunchTabs&) = 0;
   // E: V_h -> L2
-  virtual int v2l(const DevMesh&, const DevTabs&, const void* uV, void* uL, cudaStream_t) = 0;
+  virtual int v2l(const DevMesh&, const LaunchTabs&, const void* uV, void* uL, cudaStream_t) = 0;
   // facet flux moments, element-major: gam[e][f][nf][d] for the element e that sees the
   // facet as its local facet f (alpha + beta on side A, alpha - beta on side B) and, if
   // diss is not null, the facet dissipation per facet.  wL == uL means w = u.
-  virtual int facet(const DevMesh&, const DevTabs&, const void* uL, const void* wL, int l,
+  virtual int facet(const DevMesh&, const LaunchTabs&, const void* uL, const void* wL, int l,
                     const int8_t* facet_l, void* gam, double* diss, cudaStream_t) = 0;
   // volume term + facet lift + inverse mass, combined into out.  wL == uL means w = u.
-  virtual int volume(const DevMesh&, const DevTabs&, const void* uL, const void* wL,
+  virtual int volume(const DevMesh&, const LaunchTabs&, const void* uL, const void* wL,
                      const void* gam, Combine c, void* out, cudaStream_t) = 0;
   // volume kernel with the element part of R E^{-1} fused into its epilogue (w = u
   // only): writes the combined interior V_h dofs into outV and the local facet
   // functionals into lf.  Returns 0 (nothing launched) when this family has no fused
   // variant; the caller then runs volume + l2v_elem.
-  virtual int volume_l2v(const DevMesh&, const DevTabs&, const void* uL, const void* gam, void* lf,
+  virtual int volume_l2v(const DevMesh&, const LaunchTabs&, const void* uL, const void* gam, void* lf,
                          Combine c, void* outV, cudaStream_t) = 0;
   virtual bool has_fused() const = 0;
   virtual bool tensor_cores() const = 0;  // the V_h -> L2 projection runs on tensor cores
@@ -182,17 +187,17 @@ class Ops {
   // apply (ybar = cotangent of y; wL == uL means w = u and the cotangents are summed
   // into ubar, wbar unused); gamU / gamW are element-major facet-moment scratch.
   // adaptive HOPU: eta per facet with the current orders, new orders written in place
-  virtual int eta(const DevMesh&, const DevTabs&, const void* uL, int l, int8_t* facet_l,
+  virtual int eta(const DevMesh&, const LaunchTabs&, const void* uL, int l, int8_t* facet_l,
                   const EtaThresholds& th, double* eta_out, cudaStream_t) = 0;
-  virtual int v2l_pt(const DevMesh&, const DevTabs&, const void* vV, void* yL, cudaStream_t) = 0;
-  virtual int facet_adj(const DevMesh&, const DevTabs&, const void* uL, const void* wL, const void* ybar,
+  virtual int v2l_pt(const DevMesh&, const LaunchTabs&, const void* vV, void* yL, cudaStream_t) = 0;
+  virtual int facet_adj(const DevMesh&, const LaunchTabs&, const void* uL, const void* wL, const void* ybar,
                         int l, const int8_t* facet_l, void* gamU, void* gamW, cudaStream_t) = 0;
-  virtual int volume_adj(const DevMesh&, const DevTabs&, const void* uL, const void* wL, const void* ybar,
+  virtual int volume_adj(const DevMesh&, const LaunchTabs&, const void* uL, const void* wL, const void* ybar,
                          const void* gamU, const void* gamW, void* ubar, void* wbar, cudaStream_t) = 0;
   // R E^{-1} (dual = false) or E^T (dual = true), combined into outV, in two launches:
   // the element part writes interior dofs and the local facet functionals lf
   // [E][d+1][nf]; the facet part averages (or sums) the two copies into the facet dofs.
-  virtual int l2v_elem(const DevMesh&, const DevTabs&, const void* yL, bool dual, void* lf,
+  virtual int l2v_elem(const DevMesh&, const LaunchTabs&, const void* yL, bool dual, void* lf,
                        Combine c, void* outV, cudaStream_t) = 0;
   virtual int l2v_facet(const DevMesh&, const void* lf, bool dual, Combine c, void* outV,
                         cudaStream_t) = 0;

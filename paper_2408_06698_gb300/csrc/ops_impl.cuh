@@ -117,7 +117,7 @@ class OpsImpl final : public Ops {
     else return setup(k_volume_rh<D, K, MODE>, R::SMEM, 32 * R::WARPS, &g_volar_[MODE - kVolAdjU]);
   }
   template <int MODE>
-  void launch_adj(const DevMesh& m, const DevTabs& t, const void* in1, const void* ybar, const void* gam,
+  void launch_adj(const DevMesh& m, const LaunchTabs& t, const void* in1, const void* ybar, const void* gam,
                   const void* gam2, void* out, cudaStream_t st) {
     using R = VolA<MODE>;
     const int g = clamp_grid(g_volar_[MODE - kVolAdjU], (m.E + R::ELW - 1) / R::ELW, 1);
@@ -355,7 +355,7 @@ class OpsImpl final : public Ops {
 
   // The refined FP32 projection stages the sparse rows of D and, when they fit, Dinv^T per
   // CTA; as many warps per CTA as fit in ~220 KB (16, 12, 8 or 4).
-  cudaError_t configure(const DevTabs& t) override {
+  cudaError_t configure(const LaunchTabs& t) override {
     if constexpr (kRef) {
       using R = ProjRCfg<D, K>;
       csr_n_ = t.csr_n;
@@ -369,7 +369,7 @@ class OpsImpl final : public Ops {
     return cudaSuccess;
   }
 
-  int v2l(const DevMesh& m, const DevTabs& t, const void* uV, void* uL, cudaStream_t st) override {
+  int v2l(const DevMesh& m, const LaunchTabs& t, const void* uV, void* uL, cudaStream_t st) override {
     if constexpr (kTcV2lR) {
       if (tc_ == 3 && use_tc_v2l_ && t.tcv2l) {
         const int g = clamp_grid(g_v2l_tcr_, m.E, V2lTcr<D, K>::TM);
@@ -400,7 +400,7 @@ class OpsImpl final : public Ops {
     return 1;
   }
 
-  int facet(const DevMesh& m, const DevTabs& t, const void* uL, const void* wL, int l,
+  int facet(const DevMesh& m, const LaunchTabs& t, const void* uL, const void* wL, int l,
             const int8_t* facet_l, void* gam, double* diss, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (kFacR) {
@@ -431,7 +431,7 @@ class OpsImpl final : public Ops {
     return 1;
   }
 
-  int volume(const DevMesh& m, const DevTabs& t, const void* uL, const void* wL, const void* gam,
+  int volume(const DevMesh& m, const LaunchTabs& t, const void* uL, const void* wL, const void* gam,
              Combine c, void* out, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (kTcVolE) {
@@ -510,21 +510,21 @@ class OpsImpl final : public Ops {
     return vvar_ == kVolRegFused || vvar_ == kVolWarpFused || vvar_ == kVolTensor;
   }
 
-  int eta(const DevMesh& m, const DevTabs& t, const void* uL, int l, int8_t* facet_l, const EtaThresholds& th,
+  int eta(const DevMesh& m, const LaunchTabs& t, const void* uL, int l, int8_t* facet_l, const EtaThresholds& th,
           double* eta_out, cudaStream_t st) override {
     const int g = clamp_grid(g_eta_, m.NF, kWarps);
     launch(k_eta<D, K, T>, g, 32 * kWarps, eta_smem(), st, m, t, static_cast<const T*>(uL), l, facet_l, th, eta_out);
     return 1;
   }
 
-  int v2l_pt(const DevMesh& m, const DevTabs& t, const void* vV, void* yL, cudaStream_t st) override {
+  int v2l_pt(const DevMesh& m, const LaunchTabs& t, const void* vV, void* yL, cudaStream_t st) override {
     const int g = clamp_grid(g_v2lpt_, (m.E + PW::EW - 1) / PW::EW, 1);
     launch(k_v2l<D, K, T, true>, g, 32 * PW::WARPS, PW::SMEM, st, m, static_cast<const T*>(t.Dn),
            static_cast<const float4*>(nullptr), 0, 0, static_cast<const T*>(vV), static_cast<T*>(yL));
     return 1;
   }
 
-  int facet_adj(const DevMesh& m, const DevTabs& t, const void* uL, const void* wL, const void* ybar, int l,
+  int facet_adj(const DevMesh& m, const LaunchTabs& t, const void* uL, const void* wL, const void* ybar, int l,
                 const int8_t* facet_l, void* gamU, void* gamW, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (std::is_same<T, float>::value) {
@@ -560,7 +560,7 @@ class OpsImpl final : public Ops {
     return 1;
   }
 
-  int volume_adj(const DevMesh& m, const DevTabs& t, const void* uL, const void* wL, const void* ybar,
+  int volume_adj(const DevMesh& m, const LaunchTabs& t, const void* uL, const void* wL, const void* ybar,
                  const void* gamU, const void* gamW, void* ubar, void* wbar, cudaStream_t st) override {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (std::is_same<T, float>::value) {
@@ -593,7 +593,7 @@ class OpsImpl final : public Ops {
     }
   }
 
-  int volume_l2v(const DevMesh& m, const DevTabs& t, const void* uL, const void* gam, void* lf, Combine c,
+  int volume_l2v(const DevMesh& m, const LaunchTabs& t, const void* uL, const void* gam, void* lf, Combine c,
                  void* outV, cudaStream_t st) override {
     if constexpr (kTcVol) {
       if (vvar_ == kVolTensor && tensor_core_volume() && t.tcvol) {
@@ -631,7 +631,7 @@ class OpsImpl final : public Ops {
   void select_l2v(int tc) override { use_tc_l2v_ = tc != 0 && tensor_core_l2v(); }
   int selected_l2v() const override { return use_tc_l2v_ && tensor_core_l2v() ? 1 : 0; }
 
-  int l2v_elem(const DevMesh& m, const DevTabs& t, const void* yL, bool dual, void* lf, Combine c,
+  int l2v_elem(const DevMesh& m, const LaunchTabs& t, const void* yL, bool dual, void* lf, Combine c,
                void* outV, cudaStream_t st) override {
     if constexpr (kTcL2v) {
       if (!dual && use_tc_l2v_ && tc_ && t.tcl2v) {

@@ -70,14 +70,14 @@ def members(struct):
     return re.findall(r"\b(\w+)\s*=", body)
 
 
-@pytest.mark.parametrize("struct,var", [("DevMesh", "m")])
+@pytest.mark.parametrize("struct,var", [("DevMesh", "m"), ("DevTabs", "tb")])
 def test_every_array_of_a_context_is_read(struct, var):
-    """What a context uploads and passes to every launch is read by a kernel or named at a launch."""
+    """What every launch copies as an argument is read by a kernel (or named at a launch)."""
     text = "".join(re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, n)).read()) for n in sorted(os.listdir(CSRC))
                    if n.endswith(".cuh"))
     capi = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "capi.cu")).read())
     names = members(struct)
     assert len(names) >= 8
     for name in names:
-        read = re.search(rf"\b(?:{var}|t)\.{name}\b", text) or re.search(rf"c->dm\.{name}\b(?!\s*=[^=])", capi)
+        read = re.search(rf"\b{var}\.{name}\b", text) or re.search(rf"c->dm\.{name}\b(?!\s*=[^=])", capi)
         assert read, f"{struct}::{name}"
