@@ -68,7 +68,9 @@ struct FacR {
   static constexpr bool STAGE = D == 3 && K > 1;
   static constexpr size_t SMEM = size_t(O_REC + (STAGE ? WARPS * 2 * FPW * RST : 0)) * 4;
   static constexpr int REGS = 2 * NB + 3 * NF;                   // coefficients and the modal vectors
-  static constexpr int MINB = REGS <= 120 ? 3 : 2;
+  // 3D k = 2: at three CTAs an apply with w = u of 12^3 x 6 (2074 groups, 1824 warps) took two rounds and
+  // 16.2 us, at four (12 bytes spilled) 12.1; 20^3 37.1 -> 36.2 us
+  static constexpr int MINB = REGS <= 40 ? 4 : REGS <= 120 ? 3 : 2;
 };
 
 // Both sides' records of a group's facets into the warp's buffer: record r < FPW is side A of
