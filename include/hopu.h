@@ -135,7 +135,9 @@ typedef struct {
   int wind_mode;  /* hopu_wind, used by hopu_rk_substep                                    */
   int tile_hint;  /* kernel variants in the tensor-core modes: 0 = autotune (time the FP32
                      FMA and the tensor-core kernel of each family on this mesh at create
-                     and keep the faster), 1 = FMA kernels, 2 = tensor-core kernels      */
+                     and keep the faster), 1 = FMA kernels, 2 = tensor-core kernels where
+                     they exist, for the volume term variant 3 of hopu_tuning_volume
+                     (variant 6 comes from 0 or from hopu_set_volume_variant)            */
 } hopu_options;
 
 /* Build a context: validate and copy the mesh, compute FP64 geometry (Jacobians, Piola

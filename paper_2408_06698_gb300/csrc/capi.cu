@@ -777,7 +777,9 @@ thread_local std::string g_create_error;
 //  * the V_h -> L2 projection in HOPU_TF32: FMA or tensor cores;
 //  * the element back-projection in the tensor-core modes: FMA or tensor cores (timed
 //    first, so that the volume variants with a separate back-projection use the choice).
-// tile_hint 1 keeps to the FMA kernels, 2 to the tensor-core kernels where they exist.
+// tile_hint 1 keeps to the FMA kernels, 2 to the kernels with TF32 operands and the projection where
+// they exist.  kVolTensorEl is not among those of 2: its callers at k = 4 get the FMA volume kernel and
+// at k = 3 kVolTensor, as before it was there, and not whichever of two times is shorter on the day.
 // hopu_tuning / hopu_tuning_volume / hopu_tuning_l2v report the choice and the times.
 hopu_status autotune(hopu_ctx* c, int hint) {
   Ops* o = c->ops;
@@ -785,7 +787,7 @@ hopu_status autotune(hopu_ctx* c, int hint) {
   for (int v = 0; v < kVolVariants; ++v) {
     if (!o->volume_variant_ok(v)) continue;
     if (hint == 1 && (v == kVolTensor || v == kVolTensorEl)) continue;
-    if (hint == 2 && o->volume_variant_ok(kVolTensor) && v != kVolTensor) continue;
+    if (hint == 2 && (o->volume_variant_ok(kVolTensor) ? v != kVolTensor : v == kVolTensorEl)) continue;
     cand.push_back(v);
   }
   const bool tc_v2l = o->tensor_cores();
