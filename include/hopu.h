@@ -159,7 +159,8 @@ hopu_status hopu_set_stream(hopu_ctx* ctx, void* cuda_stream);
 
 /* Kernel variants in use: out2[0] for the V_h -> L2 projection (HOPU_TF32: one TF32
  * product, k_v2l_tc, 3D k <= 4 and 2D; HOPU_FP32_TC: the product of exact digits,
- * k_v2l_tcr), out2[1] for the fused STAGE volume kernel; 0 = FP32 FMA kernel, 1 =
+ * k_v2l_tcr), out2[1] for the STAGE volume kernel (variants 3 and 6 of
+ * hopu_tuning_volume are tensor-core kernels); 0 = FP32 FMA kernel, 1 =
  * tensor-core kernel.  No paper counterpart (launch tuning).                           */
 hopu_status hopu_tuning(const hopu_ctx* ctx, int* out2);
 
@@ -182,6 +183,11 @@ hopu_status hopu_tuning(const hopu_ctx* ctx, int* out2);
  * available).  No
  * paper counterpart (launch tuning).                                                  */
 hopu_status hopu_tuning_volume(const hopu_ctx* ctx, int* variant, double* ms6);
+
+/* The autotuner's times of variants 0 .. n - 1 (host, n doubles), as ms6 of
+ * hopu_tuning_volume but for every variant; -1 for those not timed.  EINVAL for a NULL
+ * pointer or n < 0.  No paper counterpart (launch tuning).                             */
+hopu_status hopu_tuning_volume_ms(const hopu_ctx* ctx, double* ms, int n);
 
 /* Override the autotuner's STAGE volume variant (the numbering of hopu_tuning_volume;
  * EINVAL for a variant this order and precision does not have).  Drops the cached substep

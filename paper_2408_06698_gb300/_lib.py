@@ -83,6 +83,7 @@ SIGNATURES = {
     "hopu_set_inlet": (c_int, [c_void_p, c_void_p, c_int64, c_void_p]),
     "hopu_tuning": (c_int, [c_void_p, POINTER(c_int)]),
     "hopu_tuning_volume": (c_int, [c_void_p, POINTER(c_int), POINTER(c_double)]),
+    "hopu_tuning_volume_ms": (c_int, [c_void_p, POINTER(c_double), c_int]),
     "hopu_set_volume_variant": (c_int, [c_void_p, c_int]),
     "hopu_tuning_l2v": (c_int, [c_void_p, POINTER(c_int), POINTER(c_double)]),
     "hopu_set_l2v_variant": (c_int, [c_void_p, c_int]),

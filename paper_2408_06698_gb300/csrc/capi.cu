@@ -1113,6 +1113,12 @@ hopu_status hopu_tuning_volume(const hopu_ctx* c, int* variant, double* ms6) {
   return HOPU_OK;
 }
 
+hopu_status hopu_tuning_volume_ms(const hopu_ctx* c, double* ms, int n) {
+  if (!c || !ms || n < 0) return HOPU_EINVAL;
+  for (int v = 0; v < n; ++v) ms[v] = v < kVolVariants ? c->vol_ms[v] : -1.0;
+  return HOPU_OK;
+}
+
 hopu_status hopu_sync(hopu_ctx* c) {
   HOPU_PRECHECK(c);
   HOPU_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -140,7 +140,7 @@ enum VolumeVariant {
   kVolTensor = 3,     // tensor-core kernel
   kVolRegTab = 4,     // register kernel with reference-gradient tables + separate back-projection
   kVolRegHalf = 5,    // register kernel, basis split over two lanes + separate back-projection
-  kVolTimed = 6,      // variants whose times hopu_tuning_volume reports
+  kVolTimed = 6,      // variants whose times hopu_tuning_volume reports (hopu_tuning_volume_ms: all)
   kVolTensorEl = 6,   // tensor-core kernel with elements along the rows + separate back-projection
   kVolVariants = 7
 };

@@ -222,7 +222,7 @@ class OpsImpl final : public Ops {
     else if (vvar_ == kVolTensor || vvar_ < 0) vvar_ = default_volume_variant();
   }
   int selected_v2l() const override { return (use_tc_v2l_ && tensor_cores()) ? 1 : 0; }
-  int selected_volume() const override { return vvar_ == kVolTensor ? 1 : 0; }
+  int selected_volume() const override { return vvar_ == kVolTensor || vvar_ == kVolTensorEl ? 1 : 0; }
   bool volume_variant_ok(int v) const override {
     switch (v) {
       case kVolRegFused: return kVolRF;

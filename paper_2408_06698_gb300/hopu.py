@@ -262,11 +262,12 @@ class Hopu:
     def tuning_volume(self) -> dict:
         """The STAGE volume kernel variant the autotuner kept and its timings (ms per launch)."""
         v = ctypes.c_int()
-        ms = (c_double * 6)()
-        self._check(self.lib.hopu_tuning_volume(self.ctx, byref(v), ms), "hopu_tuning_volume")
-        names = ["reg_fused", "reg_split", "warp_fused", "tensor", "reg_tables_split", "reg_half_split"]
+        names = ["reg_fused", "reg_split", "warp_fused", "tensor", "reg_tables_split", "reg_half_split", "tensor_rows"]
+        ms = (c_double * len(names))()
+        self._check(self.lib.hopu_tuning_volume(self.ctx, byref(v), None), "hopu_tuning_volume")
+        self._check(self.lib.hopu_tuning_volume_ms(self.ctx, ms, len(names)), "hopu_tuning_volume_ms")
         return {"variant": v.value, "name": self.VOLUME_VARIANTS.get(v.value, "?"),
-                "ms": {names[i]: ms[i] for i in range(6) if ms[i] >= 0}}
+                "ms": {n: ms[i] for i, n in enumerate(names) if ms[i] >= 0}}
 
     def set_volume_variant(self, variant: int):
         """Override the autotuner's STAGE volume variant (numbering of tuning_volume)."""
