@@ -821,7 +821,10 @@ hopu_status autotune(hopu_ctx* c, int hint) {
     const float t0 = timed_ms([&] { o->v2l(c->dm, c->dt, c->d_s1, c->d_uL, c->stream); });
     o->select(1, 0);
     const float t1 = timed_ms([&] { o->v2l(c->dm, c->dt, c->d_s1, c->d_uL, c->stream); });
-    v2l = t1 < t0;
+    // k = 1 in HOPU_FP32_TC: level alone (5^3 x 6 4.20 / 4.20 us, 10^3 4.83 / 4.44, FMA / tensor cores), but its
+    // one large CTA per SM does not start beside the neighbouring kernels: the substep of 5^3 takes 35.8 /
+    // 42.0 us, of 10^3 52.3 / 55.4, of 16^3 111.7 / 112.2
+    v2l = t1 < t0 && (c->prec != HOPU_FP32_TC || c->k > 1);
     o->select(v2l, 0);
   }
   Combine plain;

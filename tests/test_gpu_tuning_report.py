@@ -52,3 +52,9 @@ def test_times_of_the_c_call():
     assert list(ms[7:]) == [-1.0, -1.0] and ms[6] > 0 and ms[3] == -1.0
     assert g.lib.hopu_tuning_volume_ms(g.ctx, None, 9) != 0 and g.lib.hopu_tuning_volume_ms(None, ms, 9) != 0
     assert g.lib.hopu_tuning_volume_ms(g.ctx, ms, -1) != 0
+
+
+def test_projection_at_k1():
+    """The autotuner keeps the FMA projection at k = 1 in FP32_TC; tile_hint 2 still forces the other."""
+    assert _mk(12, 1, 0).tuning()["v2l"] == "fma"
+    assert _mk(12, 1, 2).tuning()["v2l"] == "tc"
