@@ -4,7 +4,8 @@
 // Work decomposition: one warp per element (projections, volume term) or per facet
 // (facet flux).  Reference tables are staged once per CTA in shared memory and the
 // grids are persistent (a multiple of the SM count), so every CTA loads them once.
-// Geometry is stored in FP64 (every precision mode) and rounded to T at use.
+// Geometry is stored in FP64 (every precision mode) and rounded to T at use (the register and
+// tensor-core kernels of the other headers read a copy rounded to FP32).
 #pragma once
 #include <type_traits>
 #include <cuda_runtime.h>

@@ -13,7 +13,11 @@
 //          a sum stays below 4 * KP * 2^14 < 2^24, so FP32 accumulation is exact in any order (from
 //          l = 3 on, where q3 enters, to 2^-24 of D_l);
 //   Y      = D_0 + 2^-8 D_1 + ... : the three small levels by Horner's rule, the first two joined by
-//          TwoSum, one rounding.  What is left out is 2^-37 of |X|max |Dinv|max.
+//          TwoSum, one rounding.
+// Two things are left out.  The larger is X's rounding: BF16 keeps 8 bits of the last digit, so a
+// functional is held to 2^-32 of the element's largest, and one below 2^-8 of that to fewer than its 24
+// bits; Y then errs by at most 2^-32 |X|max times the sum of |Dinv| over its row.  The products beyond
+// the fifth level are 2^-37 of |X|max |Dinv|max each.
 // The kernel before refined a 3xTF32 product with a compensated residual X - D Y over the nonzeros
 // of D on the CUDA cores, which took half of its time.
 //

@@ -1,5 +1,5 @@
-// a3 + a5 with the element's data in registers (FP32, STAGE wind w = u): volume term, facet
-// lift and inverse mass.
+// a3 + a5 with the element's data in registers (FP32): volume term, facet lift and inverse mass;
+// w = u first, a separate wind and the VJP below.
 //
 // A warp takes ELW = 32 / D elements and a lane owns one (element, component a) pair: the
 // coefficients c of u_a, its modal reference gradients G_c = Dm_c c (c < D, dim P^{k-1}
@@ -16,7 +16,7 @@
 // staging buffer with coalesced stores.  Differentiation lowers the degree and a trace does
 // not raise it: Dm[c][j][i] = 0 for deg phi_j >= deg phi_i and TrM[m][i] = 0 for
 // deg psi_m > deg phi_i, and both products run over the rest only.  The group's records
-// arrive by cp.async, requested one group ahead.
+// arrive by cp.async, requested one group ahead (short ones are loaded directly, DIRECT below).
 //
 // GTAB: the reference gradients at the points come from staged tables of d phi_i / d xhat_c
 // instead of the modal gradients G held in registers (d n_{b,k-1} fewer registers, more
@@ -62,6 +62,15 @@ enum VolMode {
   kVolAdjW = 3,     // VJP, cotangent of w: f = -sum_c M[c][a] sum_b u_b d^_c z_b
   kVolAdjSame = 4   // VJP with w = u: the sum of both
 };
+
+// Separate wind and VJP, many points: the test sums run in blocks of points whose partial sums
+// meet in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
+// more than a warp per element, whose points are summed pairwise; one over 46 points rounded
+// the wind's cotangent 20 % more (at k = 3 the blocks cost 5 us of 61).
+__host__ __device__ constexpr int vol_point_block(int mode, int nq) {
+  const int lim = mode == kVolWind ? 64 : (mode == kVolAdjSame ? 100 : 16);
+  return (mode != kVolSame && nq > lim) ? (nq / 8 + 1) * 2 : nq;
+}
 
 template <int D, int K, bool GTAB = false, int MODE = kVolSame>
 struct VolR {
@@ -297,12 +306,7 @@ __global__ void __launch_bounds__(32 * VolR<D, K, GTAB, MODE>::WARPS, VolR<D, K,
     // two points per pass where the registers allow it: the loads and shuffles of one overlap
     // the arithmetic of the other (an odd last point is paired with itself at weight 0)
     constexpr int XP = C::XP;
-    // Separate wind and VJP, many points: the test sums run in blocks of points whose partial sums
-    // meet in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
-    // more than a warp per element, whose points are summed pairwise; one over 46 points rounded
-    // the wind's cotangent 20 % more (at k = 3 the blocks cost 5 us of 61).
-    constexpr int QLIM = MODE == kVolWind ? 64 : (MODE == kVolAdjSame ? 100 : 16);
-    constexpr int QB = (MODE != kVolSame && NQ > QLIM) ? (NQ / 8 + 1) * 2 : NQ;
+    constexpr int QB = vol_point_block(MODE, NQ);  // points whose test sums run together
     float* yp = sY + ((act ? el : 0) * D + a) * NB;  // this lane's output entries
 #pragma unroll 1
     for (int q0 = 0; q0 < NQ; q0 += QB) {

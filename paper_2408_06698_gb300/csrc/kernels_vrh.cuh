@@ -237,12 +237,7 @@ __global__ void __launch_bounds__(32 * VolRH<D, K, MODE>::WARPS, VolRH<D, K, MOD
 #pragma unroll
     for (int j = 0; j < NP; ++j) r[j] = f2_zero();
     // two points per pass (an odd last point is paired with itself at weight 0)
-    // Separate wind and VJP, many points: the test sums run in blocks of points whose partial sums
-    // meet in the output staging buffer.  One running sum over 100 points rounded the operator 6 %
-    // more than a warp per element, whose points are summed pairwise; one over 46 points rounded
-    // the wind's cotangent 20 % more (at k = 3 the blocks cost 5 us of 61).
-    constexpr int QLIM = MODE == kVolWind ? 64 : (MODE == kVolAdjSame ? 100 : 16);
-    constexpr int QB = (MODE != kVolSame && NQ > QLIM) ? (NQ / 8 + 1) * 2 : NQ;
+    constexpr int QB = vol_point_block(MODE, NQ);  // points whose test sums run together
     float* yp = sY + ((act ? el : 0) * D + a) * NB + h;  // this lane's output entries
 #pragma unroll 1
     for (int q0 = 0; q0 < NQ; q0 += QB) {
