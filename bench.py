@@ -42,9 +42,9 @@ WORKLOAD = dict(dim=3, n=32, k=4, l=3, dt=5e-4, noise=1e-3, seed=0)
 WORKLOAD_NAME = ("3D periodic box [0,2pi]^3, 32^3 cubes x 6 tets (196,608 elements), k=4, HOPU l=3, "
                  "Taylor-Green + 1e-3 seeded noise, SSP-RK3 STAGE substeps dt=5e-4")
 BOX16 = dict(dim=3, n=16, k=3, l=2, dt=5e-4, noise=1e-3, seed=0)
-# the headline's precision mode: FP32 data; the projection's and back-projection's dense
-# products on the tensor cores in 3xTF32 (the projection refined with a compensated FP32
-# residual), the facet and volume terms on the FP32 FMA kernels; autotuned per kernel family
+# the headline's precision mode: FP32 data; on the tensor cores the projection (products of
+# exact digits in BF16), the volume term (three BF16 parts) and the back-projection (3xTF32),
+# the facet term on the FP32 FMA kernel; autotuned per kernel family
 HEADLINE_PREC = "f32_tc"
 HEADLINE_MODE = ("HOPU_FP32_TC: FP32 data; tensor-core V_h -> L2 projection (exact digit products), volume "
                  "term (three BF16 parts, six products) and back-projection (3xTF32), FP32 FMA facet kernel; "
@@ -68,7 +68,7 @@ def shape(dim, k):
     nf = comb(k + dim - 1, dim - 1)
     mv = (3 * k + 1) // 2
     mf = (3 * k + 2) // 2
-    return dict(nb=nb, nf=nf, nloc=dim * nb, nint=dim * nb - (dim + 1) * nf, nq=mv ** dim, nqf=mf ** (dim - 1),
+    return dict(nb=nb, nf=nf, nloc=dim * nb, nint=dim * nb - (dim + 1) * nf, nq=mv ** dim, nqf=mf ** (dim - 1), mf=mf,
                 nq_kernel=COMPACT_VOLUME_POINTS.get((dim, k), mv ** dim))
 
 
@@ -76,28 +76,35 @@ def algorithmic(dim, k, E, NF, tsize):
     """Per-launch algorithmic flops and bytes of each kernel family (STAGE wind: w = u).
 
     Bytes count each input/output once (coefficients, the geometry actually read, facet
-    moments, connectivity); flops count the contractions the kernels perform, the volume
-    term with the kernels' own quadrature rule (nq_kernel points).
+    moments, connectivity); flops count the contractions as the FP32 kernels perform them: the
+    volume term with the kernels' own quadrature rule (nq_kernel points), the derivative and
+    trace tables without the products that vanish by degree, the facet points of 3D by the
+    factors of the collapsed rule.
     """
     from math import comb
     s = shape(dim, k)
     nb, nf, nl, nq, nqf = s["nb"], s["nf"], s["nloc"], s["nq_kernel"], s["nqf"]
     nb1 = comb(k - 1 + dim, dim)
     d = dim
-    l = k - 1
-    nl_ = comb(l + d - 1, d - 1)
-    geo_vol = (d * d + 1) * 8                        # |det J| J^-1 and |det J| (FP64)
+    geo_vol = (d * d + 1) * tsize                    # |det J| J^-1 and |det J|
+    deg = [n for n in range(k + 1) for _ in range(comb(n + d - 1, d - 1))]    # of phi_i
+    fdeg = [n for n in range(k + 1) for _ in range(comb(n + d - 2, d - 2))]   # of psi_m
+    n_dm = sum(j < i for j in deg[:nb1] for i in deg)    # nonzeros of one derivative table
+    n_tr = sum(m <= i for m in fdeg for i in deg)        # nonzeros of one facet's trace table
     out = {}
-    # volume: modal gradients (2 d^2 nb1 nb) + per point u (2 nb d), grad u (2 nb1 d^2),
-    # W and div W (4 d^2), f (2 d^2 + 2 d), test (2 nb d) + facet lift (2 nl (d+1) nf)
+    # volume: modal gradients (2 d^2 n_dm) + per point u (2 nb d), grad u (2 nb1 d^2),
+    # W and div W (4 d^2), f (2 d^2 + 2 d), test (2 nb d) + facet lift (2 d (d+1) n_tr)
     per_q = 2 * nb * d + 2 * nb1 * d * d + 4 * d * d + 2 * d * d + 2 * d + 2 * nb * d
-    fl = E * (2 * d * d * nb1 * nb + nq * per_q + 2 * nl * (d + 1) * nf)
+    fl = E * (2 * d * d * n_dm + nq * per_q + 2 * d * (d + 1) * n_tr)
     by = E * (2 * nl * tsize + geo_vol + (d + 1) * 4) + NF * 2 * nf * d * tsize
     out["volume"] = (fl, by)
-    # facet: two traces (2 * 2 nqf nb d), P^l moments and evaluation (4 nl_ d nqf), moments
-    # of the two facet fields (2 * 2 nf d nqf)
-    fl = NF * (2 * 2 * nqf * nb * d + 4 * nl_ * d * nqf + 2 * 2 * nf * d * nqf)
-    by = NF * ((d + 1) * 8 + 2 * 4 + 2 * nf * d * tsize) + E * nl * tsize
+    # facet: two modal traces (2 * 2 d n_tr), normal parts (2 * 2 nf d), the jump, its part above l
+    # (2 d fields) and w.n to the points and alpha, beta (2 d fields) back, a field through mf rows
+    # of nf products and nqf points of k + 1 (2D: the points alone), the fluxes (5 d per point)
+    mf = s["mf"]
+    to_points = (2 * nf * mf if d == 3 else 0) + 2 * (k + 1) * nqf
+    fl = NF * (4 * d * n_tr + 4 * nf * d + (4 * d + 1) * to_points + 5 * d * nqf)
+    by = NF * ((d + 1) * tsize + 2 * 4 + 2 * nf * d * tsize) + E * nl * tsize
     out["facet"] = (fl, by)
     # v2l: gather + Dinv (2 nl^2) + Piola (2 nl d)
     out["v2l"] = (E * (2 * nl * nl + 2 * nl * d), (NF * nf + E * s["nint"]) * tsize + E * nl * tsize
