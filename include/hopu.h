@@ -194,6 +194,13 @@ hopu_status hopu_tuning_volume_ms(const hopu_ctx* ctx, double* ms, int n);
  * graph.  No paper counterpart (launch tuning).                                       */
 hopu_status hopu_set_volume_variant(hopu_ctx* ctx, int variant);
 
+/* Elements and facets that the choices by mesh size go by; 0 = this mesh's own (the
+ * default).  With a separate wind in FP32 small meshes run other kernels than large ones,
+ * which sum in another order; a context on one part of a mesh that passes the whole mesh's
+ * sizes computes the same bits as a context on the whole mesh.  Drops the cached substep
+ * graph.  EINVAL for a negative size.  No paper counterpart (launch tuning).            */
+hopu_status hopu_set_dispatch_size(hopu_ctx* ctx, int64_t n_elems, int64_t n_facets);
+
 /* The element part of the back-projection R E^{-1} (Section 2.3, the local functionals
  * D (det J Jinv y) of an L2 field y, not dual) that the autotuner kept: *tc = 1 for the
  * tensor-core kernel (k_l2v_tc: 128 elements per tile as the MMA rows, D as the B

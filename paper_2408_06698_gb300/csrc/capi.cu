@@ -1085,6 +1085,17 @@ hopu_status hopu_set_volume_variant(hopu_ctx* c, int variant) {
   return HOPU_OK;
 }
 
+hopu_status hopu_set_dispatch_size(hopu_ctx* c, int64_t n_elems, int64_t n_facets) {
+  HOPU_PRECHECK(c);
+  if (n_elems < 0 || n_facets < 0) return fail(c, HOPU_EINVAL, "set_dispatch_size: negative size");
+  c->ops->set_sizes(n_elems, n_facets);
+  if (c->gexec) {  // the captured substep uses the previous choice
+    cudaGraphExecDestroy(c->gexec);
+    c->gexec = nullptr;
+  }
+  return HOPU_OK;
+}
+
 hopu_status hopu_tuning_l2v(const hopu_ctx* c, int* tc, double* ms2) {
   if (!c || !tc) return HOPU_EINVAL;
   *tc = c->ops ? c->ops->selected_l2v() : 0;

@@ -175,6 +175,8 @@ class Ops {
   virtual bool tensor_core_volume_el() const = 0;  // ... the one with elements along the rows
   // variant choice per kernel family (autotuner): 0 = FP32 FMA kernel, 1 = tensor-core kernel
   virtual void select(int v2l_tc, int volume_tc) = 0;
+  // mesh sizes that choices by size go by (0: the mesh's own)
+  virtual void set_sizes(int64_t n_elems, int64_t n_facets) = 0;
   virtual int selected_v2l() const = 0;
   virtual int selected_volume() const = 0;
   // kernel variants of the element part of a STAGE stage (volume term, lift, inverse mass,

@@ -147,6 +147,10 @@ class OpsImpl final : public Ops {
   static constexpr int kFacAdjSmall = (D == 3 && K == 2) || (D == 2 && K == 4) ? 10 : 0;
   static constexpr int kVolAdjSmall = K == 1 ? 4 : D == 2 ? (K == 2 ? 8 : 32) : K == 2 ? 32 : 0;
   bool small(int64_t items, int per_sm) const { return items <= (int64_t)per_sm * nsm_; }
+  // the sizes these choices go by: this mesh's, or those of the mesh that it is a part of
+  int64_t size_E_ = 0, size_F_ = 0;
+  int64_t elems(const DevMesh& m) const { return size_E_ ? size_E_ : m.E; }
+  int64_t facets(const DevMesh& m) const { return size_F_ ? size_F_ : m.NF; }
   int g_facar_[2] = {1, 1};  // facet part of the VJP in FP32: w = u, separate wind
   int g_volr_ = 1, g_volrf_ = 1;
   // facet term: register-resident kernel in FP32 (every order), a warp per facet in FP64 and on small
@@ -220,6 +224,10 @@ class OpsImpl final : public Ops {
     use_tc_v2l_ = v2l_tc != 0 && tensor_cores();
     if (volume_tc != 0 && tensor_core_volume()) vvar_ = kVolTensor;
     else if (vvar_ == kVolTensor || vvar_ < 0) vvar_ = default_volume_variant();
+  }
+  void set_sizes(int64_t n_elems, int64_t n_facets) override {
+    size_E_ = n_elems;
+    size_F_ = n_facets;
   }
   int selected_v2l() const override { return (use_tc_v2l_ && tensor_cores()) ? 1 : 0; }
   int selected_volume() const override { return vvar_ == kVolTensor || vvar_ == kVolTensorEl ? 1 : 0; }
@@ -405,7 +413,7 @@ class OpsImpl final : public Ops {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (kFacR) {
       if constexpr (kFacSmall) {
-        if (wsep && small(m.NF, kFacSmall)) {
+        if (wsep && small(facets(m), kFacSmall)) {
           launch(k_facet<D, K, T, true, kFacetTab>, clamp_grid(g_fac_[1], m.NF, kWarps), 32 * kWarps, facet_smem(true), st,
               m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), l, facet_l, static_cast<T*>(gam), diss);
           return 1;
@@ -476,7 +484,7 @@ class OpsImpl final : public Ops {
     // 27 against 20 us; k = 4, 2058 elements: 37 against 39 us; 6000 elements: 70 against 53 us).
     const int g = clamp_grid(g_vol_[wsep ? 1 : 0], m.E, kWarps);
     if constexpr (kVolRW || kVolRHW) {
-      if (m.E > (int64_t)g_vol_[1] * kWarps) {
+      if (elems(m) > (int64_t)g_vol_[1] * kWarps) {
         if constexpr (kVolRW) {
           using R = VolR<D, K, false, kVolWind>;
           launch(k_volume_r<D, K, false, false, kVolWind>, clamp_grid(g_volw_, (m.E + R::ELW - 1) / R::ELW, 1),
@@ -529,7 +537,7 @@ class OpsImpl final : public Ops {
     const bool wsep = (wL != nullptr && wL != uL);
     if constexpr (std::is_same<T, float>::value) {
       if constexpr (kFacAdjSmall) {
-        if (wsep && small(m.NF, kFacAdjSmall)) {
+        if (wsep && small(facets(m), kFacAdjSmall)) {
           launch(k_facet_adj<D, K, T, true>, clamp_grid(g_fadj_, m.NF, kWarps), 32 * kWarps, facet_adj_smem(true), st,
               m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar), l, facet_l,
               static_cast<T*>(gamU), static_cast<T*>(gamW));
@@ -569,7 +577,7 @@ class OpsImpl final : public Ops {
         return 1;
       }
       if constexpr (kVolAdjSmall) {
-        if (small(m.E, kVolAdjSmall)) {
+        if (small(elems(m), kVolAdjSmall)) {
           launch(k_volume_adj<D, K, T, true>, clamp_grid(g_vadj_, m.E, kWarps), 32 * kWarps, volume_adj_smem(true), st,
               m, t, static_cast<const T*>(uL), static_cast<const T*>(wL), static_cast<const T*>(ybar),
               static_cast<const T*>(gamU), static_cast<const T*>(gamW), static_cast<T*>(ubar), static_cast<T*>(wbar));

@@ -248,6 +248,10 @@ class Hopu:
         return {"kernel": "tc" if tc.value else "fma",
                 "ms": {n: ms[i] for i, n in enumerate(("fma", "tc")) if ms[i] >= 0}}
 
+    def set_dispatch_size(self, n_elems: int = 0, n_facets: int = 0):
+        """Mesh sizes that the choice of kernels by size goes by (0: this mesh's own)."""
+        self._check(self.lib.hopu_set_dispatch_size(self.ctx, int(n_elems), int(n_facets)), "hopu_set_dispatch_size")
+
     def set_l2v_variant(self, tc: int):
         """Override the autotuner's back-projection kernel: 0 FMA, 1 tensor cores."""
         self._check(self.lib.hopu_set_l2v_variant(self.ctx, int(tc)), "hopu_set_l2v_variant")

@@ -131,6 +131,10 @@ class PartitionedHopu:
         from .hopu import Hopu
         self.parts = parts
         self.ctx = [Hopu(coords, np.asarray(elems)[p.local], rep, device=device, **opts) for p in parts]
+        # kernels as the whole mesh takes them, so that the outputs are the same bits
+        nb = facet_neighbours(elems, rep)
+        for c in self.ctx:
+            c.set_dispatch_size(nb.shape[0], int((nb >= 0).sum()) // 2 + int((nb < 0).sum()))
         self.device = self.ctx[0].device
         self.nloc = self.ctx[0].n_l2 // self.ctx[0].n_elems
         ids = lambda a: torch.as_tensor(np.asarray(a, dtype=np.int32), device=self.device)

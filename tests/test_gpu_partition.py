@@ -59,3 +59,15 @@ def test_pack_rejects_ids_outside_the_mesh():
     g.pack_elements(ids, u)
     with pytest.raises(HopuError, match="outside the mesh"):
         g.sync()
+
+
+@pytest.mark.parametrize("dim,n,k,P", [(3, 8, 3, 2), (3, 6, 4, 2), (3, 5, 5, 4), (2, 24, 3, 2), (3, 14, 1, 3)])
+def test_partition_takes_the_kernels_of_the_whole_mesh(dim, n, k, P):
+    """FP32, meshes that are large for the choice of kernels while their parts are small."""
+    test_partitioned_apply_is_bit_identical(dim, n, k, P, "f32")
+    from paper_2408_06698_gb300 import Hopu
+    from paper_2408_06698_gb300._lib import HopuError
+    m = W.periodic_box_mesh(2, 4)
+    g = Hopu(m.coords, m.elems, m.rep, k=2, l=1, prec="f32")
+    with pytest.raises(HopuError, match="negative"):
+        g.set_dispatch_size(-1, 0)
