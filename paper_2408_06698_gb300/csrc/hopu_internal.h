@@ -33,8 +33,9 @@ struct DevMesh {
 };
 
 // Device reference tables in working precision (all element-type T, 16-byte aligned) that kernels take
-// as one argument.  Every launch copies its arguments: 40 bytes more cost the 150 launches of ten
-// substeps of an 8 x 8 square 0.8 % (706 -> 711 us), so a table that only a launch names is in LaunchTabs.
+// as one argument.  Every launch copies its arguments: 24 bytes more (here and in DevMesh) cost the 150
+// launches of ten substeps of an 8 x 8 square 0.8 % (706 -> 711 us in FP64; 701 now), so a table that only
+// a launch names is in LaunchTabs.
 struct DevTabs {
   const void* Bt = nullptr;     // [nq][nbq]       phi_i(x_q), point-major, rows padded to nbq
   const void* dBt = nullptr;    // [d][nq][nbq]    d phi_i / d xhat_c (x_q), same layout as Bt
